@@ -108,32 +108,6 @@ __device__ __forceinline__ unsigned long long warp_scan_u64(unsigned long long x
     return x;
 }
 
-// Warp sum of values below 2^43 with two 32-bit warp reductions: the low
-// 16 bits of 32 lanes sum below 2^21 and the bits above below 2^32, so both
-// halves are exact.  (Degrees and line counts are below E, and the
-// PageRank priority is capped at 2^40.)  Needs all 32 lanes.
-__device__ __forceinline__ unsigned long long warp_sum_lt43(unsigned long long x) {
-    const unsigned int lo = __reduce_add_sync(0xffffffffu, (unsigned int)(x & 0xFFFFull));
-    const unsigned int hi = __reduce_add_sync(0xffffffffu, (unsigned int)(x >> 16));
-    return ((unsigned long long)hi << 16) + lo;
-}
-
-// Inclusive warp scan in 32-bit arithmetic when every lane's value is below
-// 2^27 (the warp's total then stays below 2^32), else in 64-bit.
-__device__ __forceinline__ unsigned long long warp_scan_small(unsigned long long x) {
-    if (__all_sync(0xffffffffu, x < (1ull << 27))) {
-        const int lane = threadIdx.x & 31;
-        unsigned int y = (unsigned int)x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned int t = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += t;
-        }
-        return y;
-    }
-    return warp_scan_u64(x);
-}
-
 // Counter-based mix used only for the "random route" test mode.
 __host__ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
     x ^= x >> 33; x *= 0xff51afd7ed558ccdull;
@@ -270,8 +244,10 @@ constexpr unsigned int kHubReplicas = 256;
 
 cudaError_t launch_count(const GraphDev &g, const AlgoState &st, const PartArrays &pa,
                          unsigned long long m, cudaStream_t s);
+// With ctl, the device loop's decision too: cond is the WHILE node's condition.
 cudaError_t launch_select(const GraphDev &g, const PartArrays &pa, const CostParams &cp,
-                          Summary *sum, cudaStream_t s);
+                          Summary *sum, cudaStream_t s, LoopCtl *ctl = nullptr,
+                          unsigned long long cond = 0);
 cudaError_t launch_bin(const GraphDev &g, const AlgoState &st, const PartArrays &pa,
                        const ListArrays &la, const Summary *sum, cudaStream_t s);
 
@@ -359,9 +335,6 @@ cudaError_t launch_zero_u64(unsigned long long *p, unsigned long long n, cudaStr
 // except for the tail, which is copied word by word.
 cudaError_t launch_copy_words(const unsigned int *src, unsigned int *dst, unsigned long long n,
                               const LoopCtl *loop, cudaStream_t s);
-cudaError_t launch_loop_decide(const Summary *sum, LoopCtl *ctl, unsigned long long cond_handle,
-                               cudaStream_t s);
-
 cudaError_t launch_init(const AlgoState &st, unsigned long long V, unsigned long long n_words_alloc,
                         unsigned int source, cudaStream_t s);
 cudaError_t launch_pr_finalize(const AlgoState &st, unsigned long long V, float *out,

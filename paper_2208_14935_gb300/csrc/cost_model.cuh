@@ -7,6 +7,11 @@
 
 namespace hytg {
 
+__device__ __forceinline__ unsigned long long div_up(unsigned long long x, unsigned long long d) {
+    const unsigned long long q = x / d;
+    return q + (x != q * d);
+}
+
 __device__ __forceinline__ int decide_route_counts(unsigned int p, unsigned long long Ei,
                                                    unsigned long long A, unsigned long long Ae,
                                                    unsigned long long L, const CostParams &cp) {
@@ -23,10 +28,13 @@ __device__ __forceinline__ int decide_route_counts(unsigned int p, unsigned long
     }
     if (resident) return kRouteCache;
     typedef unsigned __int128 u128;
+    // the quotients' operands are byte and line counts of one partition, far
+    // below 2^64, so they divide in 64 bits (a 128-bit division is a slow
+    // software routine); the products below are taken in 128 bits
     const unsigned long long den = cp.m * cp.MR;
-    const u128 Tef = ((u128)Ei * cp.d1 + den - 1) / den;
-    const u128 Tec = ((u128)Ae * cp.d1 + (u128)A * cp.d2 + den - 1) / den;
-    const u128 Tl = ((u128)L + cp.MR - 1) / cp.MR;
+    const u128 Tef = div_up(Ei * cp.d1, den);
+    const u128 Tec = div_up(Ae * cp.d1 + A * cp.d2, den);
+    const u128 Tl = div_up(L, cp.MR);
     // Tiz = Tl * (gamma + (1 - gamma) * Ae / Ei) = TizN / TizD
     const u128 TizN = Tl * ((u128)cp.gamma_num * Ei + (u128)(kParamDen - cp.gamma_num) * Ae);
     const u128 TizD = (u128)kParamDen * Ei;

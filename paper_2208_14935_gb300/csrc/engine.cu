@@ -296,7 +296,7 @@ struct hytg_ctx {
     cudaEvent_t ev_cstage[2] = {}, ev_clist = nullptr;
 
     // device-driven iteration loop: a graph whose WHILE node repeats one
-    // iteration (plan, k_loop_decide, bin, cache and Z relax) on the device
+    // iteration (plan, k_select, bin, cache and Z relax) on the device
     cudaStream_t s_cap = nullptr;                        // capture stream
     cudaStream_t s_cap2 = nullptr;                       // capture stream of the IF-node bodies
     // F and C iterations inside the loop: IF-node handles (host copy, device
@@ -1079,7 +1079,7 @@ hytg_status issue_plan(hytg_ctx *c, int algo, unsigned int bucket, uint32_t it, 
 // The device-sized part of an iteration once its routes are decided: k_bin,
 // then the cache relax (and its second pass) and the zero-copy relax.
 // `loop` is set when the launches are captured into the device loop's body:
-// they then run only if k_loop_decide gave the iteration to the device.
+// they then run only if k_select gave the iteration to the device.
 // part: 0 everything; while capturing the device loop's body, 1 stops after
 // k_bin and 2 issues only what follows it.
 hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStream_t s, LoopCtl *loop,
@@ -1166,7 +1166,7 @@ bool loop_fc_wanted(const hytg_ctx *c) {
 // One IF node per partition (copy the partition into the staging slot of its
 // lane, relax it, and for PageRank/PPR its second pass), chained per slot so
 // that a slot's next user starts after the previous one; one IF node for the
-// C route (gather into the compaction buffer, relax).  k_loop_decide opens the
+// C route (gather into the compaction buffer, relax).  k_select opens the
 // nodes of the partitions it routed F and the C node when C fits the buffer.
 hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::vector<cudaGraphNode_t> &after_bin) {
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
@@ -1308,8 +1308,7 @@ hytg_status capture_loop_body(hytg_ctx *c, int algo, cudaStream_t s, unsigned lo
         CK(launch_zero_u64(pa.n_act, (L.zero_end - L.n_act) / 8, s));
     }
     { ScopedTime t(c, HYTG_K_COUNT, s); CK(launch_count(g, st, pa, (unsigned long long)c->m, s)); }
-    { ScopedTime t(c, HYTG_K_COUNT, s); CK(launch_select(g, pa, cost_params(c, algo, 1), sum, s)); }
-    { ScopedTime t(c, HYTG_K_OTHER, s); CK(launch_loop_decide(sum, c->d_loop, handle, s)); }
+    { ScopedTime t(c, HYTG_K_COUNT, s); CK(launch_select(g, pa, cost_params(c, algo, 1), sum, s, c->d_loop, handle)); }
     return issue_plan_tail(c, algo, 0xFFFFFFFFu, s, c->d_loop, 1);
 }
 
@@ -1904,7 +1903,7 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
     CK(cudaGraphLaunch(c->loop_exec, c->s_main));
     CK(cudaMemcpyAsync(c->h_loop, c->d_loop, sizeof(LoopCtl), cudaMemcpyDeviceToHost, c->s_main));
     if (c->has_deadline) {
-        // past the deadline the host sets the cancel word; k_loop_decide reads
+        // past the deadline the host sets the cancel word; k_select reads
         // it at the next iteration boundary and ends the loop, so the launch
         // still ends after at most one more iteration
         for (;;) {

@@ -116,21 +116,28 @@ __global__ void k_cc_write(AlgoState st, unsigned long long V, const unsigned in
 
 // Fold the per-SM hub replicas into delta and clear them.  A block takes 32
 // consecutive hub ids; each of its 8 warps sums every 8th replica row of
-// those ids (128-byte rows, eight loads in flight), and the first warp adds
-// the 8 partial sums into delta.
+// those ids (128-byte rows), and the first warp adds the 8 partial sums into
+// delta.  Each warp's 32 rows are loaded before any is cleared: with a clear
+// behind each load the loads waited for one another (256 rows of 4,096
+// ids, 4 MiB in L2: 49 us; now 13 us together with the frontier rebuild).
 __global__ void __launch_bounds__(256) k_hub_reduce(AlgoState st) {
     __shared__ float part[8][32];
+    constexpr int kRows = kHubReplicas / 8;
     const unsigned int K = st.n_hub_rep;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (unsigned int v0 = blockIdx.x * 32u; v0 < K; v0 += gridDim.x * 32u) {
         const unsigned int v = v0 + lane;
         float s = 0.0f;
         if (v < K) {
-#pragma unroll 8
-            for (unsigned int r = wid; r < kHubReplicas; r += 8) {
-                float *p = st.hub_rep + (size_t)r * K + v;
-                s += *p;
-                *p = 0.0f;
+            float *p = st.hub_rep + (size_t)wid * K + v;
+            const size_t step = (size_t)8 * K;
+            float x[kRows];
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) x[r] = p[r * step];
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                s += x[r];
+                if (x[r] != 0.0f) p[r * step] = 0.0f;
             }
         }
         part[wid][lane] = s;
