@@ -117,11 +117,11 @@ typedef struct hytg_stats {
                                          each HYTG_K_* kind (index 12: the second pass), i.e.
                                          the wall time during which that kind was running */
     uint64_t link_sector_bytes[5];    /* host-link bytes read, counted by the kernels that
-                                         read mapped host memory (Z relaxes, C gathers): in
-                                         each 2,048-edge tile, the distinct 32-byte sectors
-                                         its edges occupy, times 32 and the arrays read; F
-                                         (and C with "compact_host"): the bytes copied;
-                                         cache 0.  Index: hytg_route */
+                                         read mapped host memory (Z relaxes, C gathers): the
+                                         32-byte sectors their edges occupy, one more where
+                                         the route's edges leave a sector and come back, times
+                                         32 and the arrays read; F (and C with "compact_host"):
+                                         the bytes copied; cache 0.  Index: hytg_route */
     uint64_t link_line_bytes[5];      /* the same count at 128-byte lines, times 128 */
     uint64_t f_reused_tasks;          /* F tasks run from a staging slot that still held
                                          their partitions ("slot_reuse"): no copy */

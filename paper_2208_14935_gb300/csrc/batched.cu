@@ -11,7 +11,7 @@
 //   PPR       *bdelta(v, s), *brank(v, s), *bmsg(v, s) (the push of seed s
 //             taken this iteration), fr32[v] mask of seeds taken.
 #include "common.cuh"
-#include "relax_tile.cuh"
+#include "edge_runs.cuh"
 
 namespace hytg {
 
@@ -202,46 +202,29 @@ __global__ void k_serve_extract(BatchState b, unsigned long long V, unsigned int
     }
 }
 
-// Multi-source BFS relax: one thread per edge; the sources of u not yet
+// Multi-source BFS relax: one lane per edge; the sources of u not yet
 // reached at v are ORed into nxt[v].
+constexpr int kBatchSteps = 4;
 __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListArrays la,
                                                              const Summary *sum, RelaxTask t) {
-    __shared__ TileSmem<true> sm;
     if (b.loop && !b.loop->work) return;
     unsigned long long kb, ke;
-    task_range(t, sum, kb, ke);
-    if (kb >= ke) return;
-    const unsigned long long t_first = kb / kTile, t_last = (ke - 1) / kTile;
-    for (unsigned long long tile = t_first + blockIdx.x; tile <= t_last; tile += gridDim.x) {
-        unsigned long long k0;
-        const int n = tile_setup<true>(sm, la, sum, t, tile, kb, ke, &k0);
-        if (t.link_ctr) count_link_reads<true>(sm, k0, n, 1u, t.link_ctr);
-        unsigned int dv[kRelaxIPT];
-        unsigned long long fv[kRelaxIPT];
+    const RouteView rv = task_view(t, sum, kb, ke);
+    LinkCount lc;
+    walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
+        unsigned int dv[kBatchSteps];
+        unsigned long long vis[kBatchSteps];
 #pragma unroll
-        for (int j = 0; j < kRelaxIPT; ++j) {
-            const int slot = threadIdx.x + j * kRelaxBlock;
-            dv[j] = kInf;
-            fv[j] = 0;
-            if (slot < n) {
-                const int i = sm.sid[slot];
-                const long long e = (long long)(k0 + slot) + sm.delta[i];
-                if (e >= 0 && (unsigned long long)e < t.src_len) {
-                    dv[j] = __ldg(t.dst + e);
-                    fv[j] = sm.pay[i];
-                } else {
-                    atomicOr(la.err, 8u);
-                }
-            }
-        }
+        for (int q = 0; q < kBatchSteps; ++q) dv[q] = ed[q].ok ? __ldg(t.dst + ed[q].e) : 0u;
 #pragma unroll
-        for (int j = 0; j < kRelaxIPT; ++j) {
-            if (dv[j] == kInf) continue;
-            const unsigned long long nb = fv[j] & ~__ldcg(&b.vis[dv[j]]);
-            if (nb) atomicOr(&b.nxt[dv[j]], nb);
+        for (int q = 0; q < kBatchSteps; ++q) vis[q] = ed[q].ok ? __ldcg(&b.vis[dv[q]]) : ~0ull;
+#pragma unroll
+        for (int q = 0; q < kBatchSteps; ++q) {
+            const unsigned long long nb = ed[q].pay & ~vis[q];
+            if (ed[q].ok && nb) atomicOr(&b.nxt[dv[q]], nb);
         }
-        __syncthreads();
-    }
+    });
+    flush_link(lc, 1u, t.link_ctr);
 }
 
 // Multi-source SSSP and batched PPR relax.  A warp loads 32 edges at once
@@ -254,216 +237,162 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
 // otherwise every lane keeps its own edge and loops over the sources active
 // at its u, so that 32 edges' loads are in flight together instead of one
 // edge's.
+__device__ __forceinline__ void mssssp_edges(const BatchState &b, unsigned int v, unsigned int w, unsigned int u,
+                                             unsigned long long f, unsigned int *overflow) {
+    const int lane = threadIdx.x & 31;
+    const unsigned int pop = __reduce_add_sync(0xffffffffu, (unsigned int)__popcll(f));
+    if (pop < b.sparse_below * 32u) {
+        // sparse masks: a lane per edge, looping over its active sources
+        unsigned long long imp = 0;
+        while (f) {
+            const unsigned int s = (unsigned int)(__ffsll((long long)f) - 1);
+            f &= f - 1;
+            const unsigned long long nd = (unsigned long long)__ldcg(bval(b, u, s)) + w;
+            if (nd >= 0xFFFFFFFEull) {
+                *overflow = 1u;
+            } else if ((unsigned int)nd < __ldcg(bval(b, v, s))) {
+                atomicMin(bval(b, v, s), (unsigned int)nd);
+                imp |= 1ull << s;
+            }
+        }
+        if (imp) atomicOr(&b.nxt[v], imp);
+        return;
+    }
+    unsigned int todo = __ballot_sync(0xffffffffu, f != 0);
+    while (todo) {
+        const int jj = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const unsigned int vj = __shfl_sync(0xffffffffu, v, jj), uj = __shfl_sync(0xffffffffu, u, jj);
+        const unsigned int wj = __shfl_sync(0xffffffffu, w, jj);
+        const unsigned long long fj = __shfl_sync(0xffffffffu, f, jj);
+        unsigned long long imp = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned int s = lane + 32 * h;
+            bool better = false;
+            if ((fj >> s) & 1ull) {
+                const unsigned long long nd = (unsigned long long)__ldcg(bval(b, uj, s)) + wj;
+                if (nd >= 0xFFFFFFFEull) {
+                    *overflow = 1u;
+                } else if ((unsigned int)nd < __ldcg(bval(b, vj, s))) {
+                    atomicMin(bval(b, vj, s), (unsigned int)nd);
+                    better = true;
+                }
+            }
+            imp |= (unsigned long long)__ballot_sync(0xffffffffu, better) << (32 * h);
+        }
+        if (lane == 0 && imp) atomicOr(&b.nxt[vj], imp);
+    }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, ListArrays la,
                                                               const Summary *sum, RelaxTask t,
                                                               unsigned int *bm,
                                                               unsigned int *overflow) {
-    __shared__ TileSmem<true> sm;
     if (b.loop && !b.loop->work) return;
     unsigned long long kb, ke;
-    task_range(t, sum, kb, ke);
-    if (kb >= ke) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned long long t_first = kb / kTile, t_last = (ke - 1) / kTile;
-    for (unsigned long long tile = t_first + blockIdx.x; tile <= t_last; tile += gridDim.x) {
-        unsigned long long k0;
-        const int n = tile_setup<true>(sm, la, sum, t, tile, kb, ke, &k0);
-        if (t.link_ctr) count_link_reads<true>(sm, k0, n, MODE == kBatchSSSP ? 2u : 1u, t.link_ctr);
-        const int per_warp = kTile / (kRelaxBlock / 32);           // 256 slots
-        for (int c = wid * per_warp; c < (wid + 1) * per_warp && c < n; c += 32) {
-            const int slot = c + lane;
-            unsigned int dj = kInf, wj = 0, uj = 0;
-            unsigned long long fj = 0;
-            if (slot < n) {
-                const int i = sm.sid[slot];
-                const long long e = (long long)(k0 + slot) + sm.delta[i];
-                if (e >= 0 && (unsigned long long)e < t.src_len) {
-                    dj = __ldg(t.dst + e);
-                    if (MODE == kBatchSSSP) wj = __ldg(t.w + e);
-                    uj = sm.vid[i];
-                    fj = sm.pay[i];
-                } else {
-                    atomicOr(la.err, 8u);
-                }
+    const RouteView rv = task_view(t, sum, kb, ke);
+    LinkCount lc;
+    walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
+        unsigned int dv[kBatchSteps], wv[kBatchSteps];
+#pragma unroll
+        for (int q = 0; q < kBatchSteps; ++q) {
+            dv[q] = wv[q] = 0;
+            if (ed[q].ok) {
+                dv[q] = __ldg(t.dst + ed[q].e);
+                if (MODE == kBatchSSSP) wv[q] = __ldg(t.w + ed[q].e);
             }
-            if (dj == kInf) fj = 0;
+        }
+#pragma unroll
+        for (int q = 0; q < kBatchSteps; ++q) {
+            const unsigned long long f = ed[q].ok ? ed[q].pay : 0ull;
             if (MODE == kBatchPPR) {
                 // a lane per edge, a frame's 8 seeds per pair of vector reductions
-                const unsigned int m = (unsigned int)fj;
-                if (m) {
-                    atomicOr(&bm[dj >> 5], 1u << (dj & 31));
-                    ppr_push_vec(b, uj, dj, m);
+                if (f) {
+                    atomicOr(&bm[dv[q] >> 5], 1u << (dv[q] & 31));
+                    ppr_push_vec(b, ed[q].vid, dv[q], (unsigned int)f);
                 }
-                continue;
-            }
-            unsigned int pop = __popcll(fj);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) pop += __shfl_xor_sync(0xffffffffu, pop, o);
-            if (pop < b.sparse_below * 32u) {
-                // sparse masks: a lane per edge, looping over its active sources
-                if (MODE == kBatchSSSP) {
-                    unsigned long long m = fj, imp = 0;
-                    while (m) {
-                        const unsigned int s = (unsigned int)(__ffsll((long long)m) - 1);
-                        m &= m - 1;
-                        const unsigned long long nd = (unsigned long long)__ldcg(bval(b, uj, s)) + wj;
-                        if (nd >= 0xFFFFFFFEull) {
-                            *overflow = 1u;
-                        } else if ((unsigned int)nd < __ldcg(bval(b, dj, s))) {
-                            atomicMin(bval(b, dj, s), (unsigned int)nd);
-                            imp |= 1ull << s;
-                        }
-                    }
-                    if (imp) atomicOr(&b.nxt[dj], imp);
-                }
-                continue;
-            }
-            const int cnt = min(32, n - c);
-            for (int jj = 0; jj < cnt; ++jj) {
-                const unsigned int v = __shfl_sync(0xffffffffu, dj, jj);
-                if (v == kInf) continue;                               // warp-uniform
-                const unsigned int u = __shfl_sync(0xffffffffu, uj, jj);
-                const unsigned long long f = __shfl_sync(0xffffffffu, fj, jj);
-                if (MODE == kBatchSSSP) {
-                    const unsigned int w = __shfl_sync(0xffffffffu, wj, jj);
-                    unsigned long long imp = 0;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const unsigned int s = lane + 32 * h;
-                        bool better = false;
-                        if ((f >> s) & 1ull) {
-                            const unsigned long long nd = (unsigned long long)__ldcg(bval(b, u, s)) + w;
-                            if (nd >= 0xFFFFFFFEull) {
-                                *overflow = 1u;
-                            } else if ((unsigned int)nd < __ldcg(bval(b, v, s))) {
-                                atomicMin(bval(b, v, s), (unsigned int)nd);
-                                better = true;
-                            }
-                        }
-                        imp |= (unsigned long long)__ballot_sync(0xffffffffu, better) << (32 * h);
-                    }
-                    if (lane == 0 && imp) atomicOr(&b.nxt[v], imp);
-                }
+            } else {
+                if (__any_sync(0xffffffffu, f != 0)) mssssp_edges(b, dv[q], wv[q], ed[q].vid, f, overflow);
             }
         }
-        __syncthreads();
-    }
+    });
+    flush_link(lc, MODE == kBatchSSSP ? 2u : 1u, t.link_ctr);
 }
 
-// Batched PPR second pass over a resident range [vlo, vhi) whose edges sit in
-// `dst` (CSR edge shift at index 0), Sec. VI-A: the seeds whose residual at a
-// vertex of the range rose above eps during this iteration are taken again
-// and pushed along the still-resident edges.  k_bsp_take: a warp per 32
-// consecutive vertices, lanes are seeds; each vertex's taken seeds go to
-// sc.pay[v] (a 32-bit mask), the vertex's taken bit to sc.mask, and the
-// owners of the 256-edge chunks starting in its list to sc.owner.  The
-// residual is read and then subtracted with a reduction, so pushes that land
-// meanwhile (other streams' relaxes) stay for later.
-__global__ void k_bsp_take(BatchState b, const unsigned long long *off, unsigned long long vlo,
-                           unsigned long long vhi, unsigned int K, float damping, float eps,
-                           SecondPassScratch sc, unsigned long long *edges_out) {
+// Batched PPR second pass over a resident range [vlo, vhi) (Sec. VI-A): the
+// seeds whose residual at a vertex of the range rose above eps during this
+// iteration are taken again, the vertices listed with their masks of taken
+// seeds, and k_relax_mswarp pushes the list from the resident copy.  A warp
+// takes 32 consecutive vertices, lanes are seeds; eight vertices' residuals
+// are read together (one at a time, each waited for the one before: a
+// dependent read of 128 bytes per vertex).  The residual is read and then
+// subtracted with a reduction, so pushes that land meanwhile (other streams'
+// relaxes) stay for later.
+__global__ void __launch_bounds__(kRelaxBlock) k_bsp_take(BatchState b, const unsigned long long *off,
+                                                          SecondPassRange r, ListArrays la, unsigned int K,
+                                                          float damping, float eps) {
     if (b.loop && !b.loop->work) return;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned int lt_mask = (1u << lane) - 1u;
     const bool has = lane < (int)K && b.delta[lane >> 3] != nullptr;
     unsigned long long done = 0;
-    const unsigned long long nw = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    for (unsigned long long base = vlo + (((blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5) << 5);
-         base < vhi; base += nw * 32) {
-        unsigned int bits = 0;
-        for (int q = 0; q < 32 && base + q < vhi; ++q) {
-            const unsigned long long v = base + q;
-            const unsigned long long e0 = off[v], deg = off[v + 1] - e0;
-            const float dl = has ? __ldcg(bdelta(b, v, lane)) : 0.0f;
-            const bool act = has && dl > eps;
-            if (act) {
-                atomicAdd(bdelta(b, v, lane), -dl);
-                *brank(b, v, lane) += dl;
-            }
-            const unsigned int seeds = __ballot_sync(0xffffffffu, act) & (deg ? 0xffffffffu : 0u);
-            // the vector push adds whole frames: the seeds not taken carry 0
-            // (this task's relax of v, the only reader of v's old messages,
-            // has finished on this stream)
-            if (seeds && has) *bmsg(b, v, lane) = act ? damping * dl / (float)deg : 0.0f;
-            if (lane == 0) sc.pay[v] = seeds;
-            if (seeds) {
-                bits |= 1u << q;
-                done += (unsigned long long)__popc(seeds) * deg;
-            }
-            // every chunk that starts in v's list has v as its owner, taken or
-            // not: the push starts its owner search there
-            if (deg) {
-                const unsigned long long c_beg = (e0 + kSpChunk - 1) / kSpChunk, c_end = (e0 + deg - 1) / kSpChunk + 1;
-                for (unsigned long long c = c_beg + lane; c < c_end; c += 32) sc.owner[c] = (unsigned int)v;
-            }
+    for (unsigned long long b0 = r.vlo + blockIdx.x * (unsigned long long)kRelaxBlock; b0 < r.vhi;
+         b0 += gridDim.x * (unsigned long long)kRelaxBlock) {
+        const unsigned long long base = b0 + 32ull * wid, v = base + lane;
+        unsigned long long o0 = 0, deg = 0;
+        if (v < r.vhi) {
+            o0 = off[v];
+            deg = off[v + 1] - o0;
         }
-        if (lane == 0) sc.mask[base >> 5] = bits;
-    }
-    if (lane == 0 && done) atomicAdd(edges_out, done);
-}
-
-// Batched PPR second-pass push: whole 256-edge chunks per warp, the owner of
-// each edge found among a window of 32 consecutive vertices; a lane keeps its
-// edge and loops over the seeds taken at the edge's source.
-__global__ void k_bsp_push(BatchState b, const unsigned long long *off, const unsigned int *dst,
-                           long long shift, unsigned long long src_len, unsigned long long vlo,
-                           unsigned long long vhi, unsigned long long E0, unsigned long long E1,
-                           SecondPassScratch sc, unsigned int *bm, unsigned int *err) {
-    if (b.loop && !b.loop->work) return;
-    if (E1 <= E0) return;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-    const unsigned long long c_first = E0 / kSpChunk, c_last = (E1 - 1) / kSpChunk;
-    for (unsigned long long c = c_first + ((blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5);
-         c <= c_last; c += nwarps) {
-        const unsigned long long k0 = c * kSpChunk > E0 ? c * kSpChunk : E0;
-        const unsigned long long k1 = (c + 1) * kSpChunk < E1 ? (c + 1) * kSpChunk : E1;
-        unsigned long long u0 = c * kSpChunk >= E0 ? (unsigned long long)sc.owner[c] : vlo;
-        if (u0 < vlo || u0 >= vhi) {
-            if (lane == 0) atomicOr(err, 32u);
-            continue;
-        }
-        unsigned long long kb = k0;
-        while (kb < k1) {
-            const unsigned long long u = u0 + lane;
-            const unsigned long long su = u < vhi ? off[u] : E1;
-            const unsigned long long ue = u0 + 32 < vhi ? u0 + 32 : vhi;
-            const unsigned long long wend_all = off[ue];
-            const bool tk = u < vhi && ((sc.mask[u >> 5] >> (u & 31)) & 1u);
-            const unsigned int seeds = tk ? sc.pay[u] : 0u;
-            const unsigned int tmask = __ballot_sync(0xffffffffu, tk);
-            const unsigned long long wend = wend_all < k1 ? wend_all : k1;
-            if (tmask) {
-                for (unsigned long long r0 = kb; r0 < wend; r0 += 32) {
-                    const unsigned long long k = r0 + lane;
-                    int own = 0;
+        unsigned int mine = 0;                      // seeds taken at this lane's vertex
 #pragma unroll
-                    for (int step = 16; step > 0; step >>= 1) {
-                        const unsigned long long cand = __shfl_sync(0xffffffffu, su, own + step);
-                        if (cand <= k) own += step;
-                    }
-                    unsigned int m = __shfl_sync(0xffffffffu, seeds, own);
-                    if (k >= wend) m = 0;
-                    if (m) {
-                        const long long i = (long long)k - shift;
-                        if (i < 0 || (unsigned long long)i >= src_len) {
-                            atomicOr(err, 16u);
-                        } else {
-                            const unsigned int w = __ldg(dst + i);
-                            atomicOr(&bm[w >> 5], 1u << (w & 31));
-                            ppr_push_vec(b, u0 + own, w, m);
-                        }
-                    }
+        for (int g = 0; g < 32; g += 8) {
+            float dl[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                dl[q] = has && base + g + q < r.vhi ? __ldcg(bdelta(b, base + g + q, lane)) : 0.0f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const bool act = dl[q] > eps;
+                const unsigned int seeds = __ballot_sync(0xffffffffu, act);
+                if (seeds == 0) continue;           // warp-uniform
+                const unsigned long long u = base + g + q, du = __shfl_sync(0xffffffffu, deg, g + q);
+                if (act) {
+                    atomicAdd(bdelta(b, u, lane), -dl[q]);
+                    *brank(b, u, lane) += dl[q];
                 }
+                if (du == 0) continue;
+                // the vector push adds whole frames: the seeds not taken carry 0
+                // (this task's relax of u, the only reader of u's old messages,
+                // has finished on this stream)
+                if (has) *bmsg(b, u, lane) = act ? damping * dl[q] / (float)du : 0.0f;
+                if (lane == g + q) mine = seeds;
             }
-            if (wend <= kb && ue >= vhi) {
-                if (lane == 0) atomicOr(err, 32u);
-                break;
+        }
+        done += (unsigned long long)__popc(mine) * deg;
+        const unsigned long long d = mine ? deg : 0ull, incl = warp_scan_u64(d);
+        const unsigned int bal = __ballot_sync(0xffffffffu, d > 0);
+        unsigned long long block_edges;
+        const ListPlace at = block_reserve(__popc(bal), __shfl_sync(0xffffffffu, incl, 31), r.cursor, block_edges);
+        if (d) {
+            const unsigned long long idx = at.entry + __popc(bal & lt_mask), eb = at.edge + incl - d;
+            const unsigned long long t1 = (eb + d - 1) / kTile;
+            if (idx >= r.vhi - r.vlo || r.tbase + t1 >= la.cap_tiles) {
+                atomicOr(la.err, 16u);
+            } else {
+                la.ebase[r.vlo + idx] = eb;
+                la.soff[r.vlo + idx] = o0;
+                la.pay64[r.vlo + idx] = mine;
+                la.vid[r.vlo + idx] = (unsigned int)v;
+                for (unsigned long long t = (eb + kTile - 1) / kTile; t <= t1; ++t)
+                    la.tile_first[r.tbase + t] = (unsigned int)idx;
             }
-            if (wend > kb) kb = wend;
-            u0 += 32;
         }
     }
+    done = warp_sum_u64(done);
+    if (lane == 0 && done) atomicAdd(r.edges_out, done);
 }
 
 __global__ void k_b_out(BatchState b, unsigned long long V, unsigned int K, const unsigned int *perm,
@@ -541,9 +470,8 @@ cudaError_t launch_relax_batched(const BatchState &b, const ListArrays &la, cons
                                  unsigned int *overflow, cudaStream_t s) {
     unsigned int grid = (unsigned int)grid_cap;
     if (!t.device_sized && !t.dev_edge) {
-        if (t.k_begin >= t.k_end) return cudaSuccess;
-        const unsigned long long tiles = (t.k_end - 1) / kTile - t.k_begin / kTile + 1;
-        if (tiles < grid) grid = (unsigned int)tiles;
+        if (t.k_begin >= t.k_end) return t.sp_reset ? cudaMemsetAsync(t.sp_reset, 0, 8, s) : cudaSuccess;
+        grid = run_blocks(t.k_begin, t.k_end, grid);
     }
     if (b.mode == kBatchBFS) k_relax_msbfs<<<grid, kRelaxBlock, 0, s>>>(b, la, sum, t);
     else if (b.mode == kBatchSSSP)
@@ -553,24 +481,15 @@ cudaError_t launch_relax_batched(const BatchState &b, const ListArrays &la, cons
 }
 
 cudaError_t launch_second_pass_batched(const BatchState &b, const unsigned long long *off,
-                                       const unsigned int *dst, long long shift,
-                                       unsigned long long src_len, unsigned long long vlo,
-                                       unsigned long long vhi, unsigned long long E0,
-                                       unsigned long long E1, unsigned int K, float damping, float eps,
-                                       const SecondPassScratch &sc, unsigned long long *edges_out,
-                                       unsigned int *bm, unsigned int *err, cudaStream_t s) {
-    if (vhi <= vlo) return cudaSuccess;
-    if ((vlo & 31) || b.mode != kBatchPPR) return cudaErrorInvalidValue;
-    const unsigned long long cap = 8ull * device_sms();
-    unsigned long long tb = (vhi - vlo + 255) / 256;          // 8 warps of 32 vertices per block
-    if (tb > cap) tb = cap;
-    const unsigned long long chunks = E1 > E0 ? (E1 - 1) / kSpChunk - E0 / kSpChunk + 1 : 0ull;
-    unsigned long long pb = (chunks + 7) / 8;
-    if (pb > cap) pb = cap;
-    if (pb == 0) pb = 1;
-    k_bsp_take<<<(unsigned int)tb, 256, 0, s>>>(b, off, vlo, vhi, K, damping, eps, sc, edges_out);
-    k_bsp_push<<<(unsigned int)pb, 256, 0, s>>>(b, off, dst, shift, src_len, vlo, vhi, E0, E1, sc, bm, err);
-    return cudaGetLastError();
+                                       const SecondPassRange &r, const ListArrays &la, const Summary *sum,
+                                       unsigned int K, float damping, float eps, unsigned int *bm,
+                                       cudaStream_t s) {
+    if (r.vhi <= r.vlo) return cudaSuccess;
+    if ((r.vlo & 31) || b.mode != kBatchPPR || r.vhi - r.vlo > kSpEntries || r.E1 - r.E0 > kSpEdgesMax)
+        return cudaErrorInvalidValue;
+    k_bsp_take<<<sp_take_blocks(r.vhi - r.vlo, kRelaxBlock), kRelaxBlock, 0, s>>>(b, off, r, la, K, damping, eps);
+    return launch_relax_batched(b, la, sum, sp_push_task(r),
+                                r.E1 > r.E0 ? (int)run_blocks(0, r.E1 - r.E0, 8 * device_sms()) : 1, bm, nullptr, s);
 }
 
 cudaError_t launch_serve_admit(const BatchState &b, unsigned long long V, unsigned int slot,

@@ -16,10 +16,14 @@ constexpr int kRouteNone = 0, kRouteCache = 1, kRouteF = 2, kRouteC = 3, kRouteZ
 // kernels set the bits of changed vertices for the next iteration.
 constexpr int kBitmapPadWords = 32;
 
-// Edge tiles of the load-balanced relax kernels.
+// Route edges per entry of the tile index (the list entry that owns the tile's
+// first edge) and at most per run, the unit of work of a warp of the relax kernels.
 constexpr int kRelaxBlock = 256;
-constexpr int kRelaxIPT = 8;
-constexpr int kTile = kRelaxBlock * kRelaxIPT;   // 2048 edges per tile
+constexpr int kTile = 2048;
+constexpr int kRunShift = 8, kRun = 1 << kRunShift;
+
+// The compaction buffer is a multiple of this many edges.
+constexpr int kCompactUnit = 2048;
 
 constexpr int kSelectBlock = 512;    // 128 registers per thread: the per-route sums stay in registers
 
@@ -270,7 +274,16 @@ struct RelaxTask {
     // route's edge space, its active edges and its first list entry, read on
     // the device where k_select and k_bin left them (nullptr: host bounds)
     const unsigned long long *dev_edge, *dev_len, *dev_entry;
+    // A second pass's push: its list is [sp_rbase, ...) of the second-pass
+    // arrays, sized by the range's cursor (nullptr: a route's list)
+    const unsigned long long *sp_cursor;
+    unsigned long long sp_rbase, sp_tbase;
+    // The cursor of the second pass that follows this launch, cleared by it
+    unsigned long long *sp_reset;
 };
+
+// Cursor of a second pass's list: entries in the low 30 bits, edges above.
+constexpr unsigned long long kSpEntries = (1ull << 30) - 1, kSpEdgesMax = (1ull << 34) - 1;
 
 cudaError_t launch_relax(const AlgoState &st, const ListArrays &la, const Summary *sum,
                          const RelaxTask &t, int grid_cap, cudaStream_t s);
@@ -279,29 +292,27 @@ cudaError_t launch_relax_pair(const AlgoState &st, const ListArrays &la, const S
                               const RelaxTask &ta, const RelaxTask &tb, int grid, cudaStream_t s);
 // Second pass (Sec. VI-A) over vertices [vlo, vhi) (vlo a multiple of 32)
 // whose edges [E0, E1) are resident in dst / w (CSR edge shift at index 0):
-// a take launch and an edge-balanced push launch.  Scratch shared by every
-// second pass of a run (their vertex and edge ranges never overlap):
-constexpr unsigned long long kSpChunk = 256;      // edges per push chunk
-struct SecondPassScratch {
-    unsigned int *owner;    // per CSR chunk of kSpChunk edges: vertex owning its first edge
-    unsigned int *pay;      // per vertex: value it pushes (taken vertices)
-    unsigned int *mask;     // per 32 vertices: bit set when taken
+// a take launch, which lists the vertices it takes as k_bin lists a route's,
+// and a relax over that list.  The list's entries lie at [vlo, vhi) and its
+// tiles from `tbase` of arrays shared by every second pass of a run, whose
+// ranges never overlap; *cursor must be zero (see RelaxTask::sp_reset).
+struct SecondPassRange {
+    unsigned long long vlo, vhi, E0, E1;
+    unsigned long long tbase;            // first tile of the range's slice
+    unsigned long long *cursor;          // packed entries and edges of its list
+    unsigned long long *edges_out;       // statistics: edges taken
+    const unsigned int *dst, *w;
+    long long shift;
+    unsigned long long src_len;
 };
-cudaError_t launch_second_pass(const AlgoState &st, const unsigned long long *off,
-                               const unsigned int *dst, const unsigned int *w, long long shift,
-                               unsigned long long src_len, unsigned long long vlo,
-                               unsigned long long vhi, unsigned long long E0, unsigned long long E1,
-                               const SecondPassScratch &sc, unsigned long long *edges_out,
-                               unsigned int *err, cudaStream_t s);
-// Batched PPR: the second pass (Sec. VI-A) over a resident range, taking
-// each seed whose residual rose above eps again (K seeds).
+cudaError_t launch_second_pass(const AlgoState &st, const unsigned long long *off, const SecondPassRange &r,
+                               const ListArrays &la, const Summary *sum, cudaStream_t s);
+// Batched PPR: the second pass over a resident range, taking each seed whose
+// residual rose above eps again (K seeds).
 cudaError_t launch_second_pass_batched(const BatchState &b, const unsigned long long *off,
-                                       const unsigned int *dst, long long shift,
-                                       unsigned long long src_len, unsigned long long vlo,
-                                       unsigned long long vhi, unsigned long long E0,
-                                       unsigned long long E1, unsigned int K, float damping, float eps,
-                                       const SecondPassScratch &sc, unsigned long long *edges_out,
-                                       unsigned int *bm, unsigned int *err, cudaStream_t s);
+                                       const SecondPassRange &r, const ListArrays &la, const Summary *sum,
+                                       unsigned int K, float damping, float eps, unsigned int *bm,
+                                       cudaStream_t s);
 cudaError_t launch_gather(const ListArrays &la, const Summary *sum, const RelaxTask &t,
                           unsigned int *out_dst, unsigned int *out_w, int grid_cap,
                           cudaStream_t s, const LoopCtl *loop = nullptr);

@@ -181,8 +181,12 @@ struct hytg_ctx {
     double *d_bsums = nullptr;
     unsigned long long *d_alive = nullptr;
     unsigned long long *d_sp = nullptr;                  // second-pass edge counters (kSpSlots)
-    unsigned int *d_sp_owner = nullptr;                  // second pass: owner of each kSpChunk-edge chunk
-    unsigned int *d_sp_mask = nullptr;                   // second pass: taken bits (one word per 32 vertices)
+    // second passes: lists of the vertices they take (entries at the
+    // vertices' own places), tile index and one cursor per partition;
+    // allocated by the first run that has them
+    unsigned long long *d_sp_ebase = nullptr, *d_sp_soff = nullptr, *d_sp_pay64 = nullptr, *d_sp_cursor = nullptr;
+    unsigned int *d_sp_tiles = nullptr, *d_sp_vid = nullptr;
+    uint64_t sp_tiles = 0;
     uint32_t sp_launches = 0;                            // host-issued second passes this run
     unsigned long long *d_link_ctr = nullptr;            // per route {sectors, lines} read from host memory
     // serving (continuous batching over the batched state)
@@ -423,8 +427,8 @@ void free_graph(hytg_ctx *c) {
     dfree(c->d_out); dfree(c->d_ebase); dfree(c->d_soff); dfree(c->d_pay); dfree(c->d_tiles);
     dfree(c->d_part_wb); dfree(c->d_part_eb); dfree(c->d_sumbuf); dfree(c->d_perm); dfree(c->d_round_part);
     dfree(c->d_hub_rep);
-    dfree(c->d_sp_owner);
-    dfree(c->d_sp_mask);
+    dfree(c->d_sp_ebase); dfree(c->d_sp_soff); dfree(c->d_sp_pay64); dfree(c->d_sp_vid);
+    dfree(c->d_sp_cursor); dfree(c->d_sp_tiles);
     c->n_hub_rep = 0;
     dfree(c->bs.fr); dfree(c->bs.vis); dfree(c->bs.nxt); dfree(c->bs.fr32);
     dfree(c->d_pay64); dfree(c->d_vid); dfree(c->d_bout);
@@ -605,6 +609,7 @@ hytg_status upload_partitions(hytg_ctx *c) {
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
     free_loop_graph(c);             // its body holds the arrays freed here
     dfree(c->d_part_wb); dfree(c->d_part_eb); dfree(c->d_sumbuf); dfree(c->d_round_part);
+    dfree(c->d_sp_cursor); dfree(c->d_sp_tiles);    // sized by the partitions
     for (int i = 0; i < 2; ++i) {
         if (c->h_sumbuf[i]) cudaFreeHost(c->h_sumbuf[i]);
         c->h_sumbuf[i] = nullptr;
@@ -656,7 +661,7 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     n.part_edges = pe;
     const uint64_t eb = 4ull * n_arrays;
     const uint64_t min_slot = std::max<uint64_t>(c->max_part_edges, 1);
-    const uint64_t compact_min = std::max<uint64_t>(kTile, 1);
+    const uint64_t compact_min = kCompactUnit;
     if (B < (min_slot + compact_min) * eb)
         return fail(c, HYTG_ERR_BUDGET, "device budget " + std::to_string(B) +
                                             " B is below one staging slot of the largest partition (" +
@@ -672,8 +677,8 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     uint64_t rem = B - n_slots * slot_edges * eb;
     uint64_t compact_edges = std::max<uint64_t>(compact_min, (uint64_t)(B * c->compact_frac) / eb);
     compact_edges = std::min<uint64_t>(compact_edges, rem / eb);
-    compact_edges = compact_edges / kTile * kTile;
-    if (compact_edges < (uint64_t)kTile) compact_edges = kTile;
+    compact_edges = compact_edges / kCompactUnit * kCompactUnit;
+    if (compact_edges < (uint64_t)kCompactUnit) compact_edges = kCompactUnit;
     rem -= compact_edges * eb;
     // cache: largest prefix of whole partitions that fits
     uint32_t n_cached = 0;
@@ -798,16 +803,6 @@ GraphDev graph_dev(hytg_ctx *c) {
     return g;
 }
 
-// The second passes' scratch; their push values live in d_out, which holds
-// nothing until the run's finalisation writes the result.
-SecondPassScratch sp_scratch(hytg_ctx *c) {
-    SecondPassScratch sc;
-    sc.owner = c->d_sp_owner;
-    sc.pay = (unsigned int *)c->d_out;
-    sc.mask = c->d_sp_mask;
-    return sc;
-}
-
 ListArrays list_arrays(hytg_ctx *c) {
     ListArrays l;
     l.ebase = c->d_ebase;
@@ -819,6 +814,22 @@ ListArrays list_arrays(hytg_ctx *c) {
     l.err = c->d_err;
     l.pay64 = c->d_pay64;
     l.vid = c->d_vid;
+    return l;
+}
+
+// The second passes' lists; their push values live in d_out, which holds
+// nothing until the run's finalisation writes the result.
+ListArrays sp_list_arrays(hytg_ctx *c) {
+    ListArrays l;
+    l.ebase = c->d_sp_ebase;
+    l.soff = c->d_sp_soff;
+    l.pay = (unsigned int *)c->d_out;
+    l.tile_first = c->d_sp_tiles;
+    l.cap_entries = c->V;
+    l.cap_tiles = c->sp_tiles;
+    l.err = c->d_err;
+    l.pay64 = c->d_sp_pay64;
+    l.vid = c->d_sp_vid;
     return l;
 }
 
@@ -910,20 +921,80 @@ bool second_pass_on(const hytg_ctx *c, int algo) {
     return c->two_pass == 2 || algo == kPR || algo == kPPR;
 }
 
-// The second pass over a resident range, single-source or batched PPR.
-cudaError_t second_pass_any(hytg_ctx *c, const AlgoState &st, const unsigned int *dst, const unsigned int *w,
-                            long long shift, unsigned long long src_len, unsigned long long vlo,
-                            unsigned long long vhi, unsigned long long E0, unsigned long long E1,
-                            unsigned long long *ctr, cudaStream_t s) {
-    if (c->batch_mode == kBatchPPR) {
-        BatchState b = c->bs;
-        b.loop = st.loop;
-        return launch_second_pass_batched(b, c->d_off, dst, shift, src_len, vlo, vhi, E0, E1, c->batch_K,
-                                          (float)c->pr_damping, (float)c->pr_eps, sp_scratch(c), ctr,
-                                          st.bm_cur, c->d_err, s);
+// Arrays of the second passes, allocated by the first run that has them and
+// kept with the graph (vertex-side data, outside the budget).
+hytg_status ensure_second_pass(hytg_ctx *c, int algo) {
+    if (!second_pass_on(c, algo)) return HYTG_OK;
+    const uint64_t N = c->part_vb.size() - 1;
+    if (!c->d_sp_ebase) {
+        CK(cudaMalloc(&c->d_sp_ebase, c->V * 8));
+        CK(cudaMalloc(&c->d_sp_soff, c->V * 8));
+        c->vertex_bytes += c->V * 16;
     }
-    return launch_second_pass(st, c->d_off, dst, w, shift, src_len, vlo, vhi, E0, E1, sp_scratch(c), ctr,
-                              c->d_err, s);
+    if (!c->d_sp_cursor) {
+        c->sp_tiles = c->E / kTile + N + 2;
+        CK(cudaMalloc(&c->d_sp_tiles, c->sp_tiles * 4));
+        CK(cudaMalloc(&c->d_sp_cursor, N * 8));
+        CK(cudaMemset(c->d_sp_cursor, 0, N * 8));
+    }
+    if (c->batch_mode == kBatchPPR && !c->d_sp_pay64) {
+        CK(cudaMalloc(&c->d_sp_pay64, c->V * 8));
+        CK(cudaMalloc(&c->d_sp_vid, c->V * 4));
+    }
+    return HYTG_OK;
+}
+
+// Partitions [i, j) of one second-pass list: as many as the packed cursor
+// holds (2^30 vertices, 2^34 edges), in practice all.
+uint32_t sp_list_end(const hytg_ctx *c, uint32_t i, uint32_t end) {
+    uint32_t j = i + 1;
+    while (j < end && c->part_vb[j + 1] - c->part_vb[i] <= kSpEntries &&
+           c->part_eb[j + 1] - c->part_eb[i] <= kSpEdgesMax)
+        ++j;
+    return j;
+}
+
+// The cursor that the launch before the second pass of partitions [i, ...)
+// clears.  A range of several lists clears the others itself.
+unsigned long long *sp_first_cursor(const hytg_ctx *c, uint32_t i) { return c->d_sp_cursor + i; }
+
+// The second pass over the resident partitions [i, end), single-source or
+// batched PPR.
+cudaError_t second_pass_any(hytg_ctx *c, const AlgoState &st, const unsigned int *dst, const unsigned int *w,
+                            long long shift, unsigned long long src_len, uint32_t i, uint32_t end,
+                            unsigned long long *ctr, cudaStream_t s) {
+    const ListArrays la = sp_list_arrays(c);
+    const Summary *sum = (const Summary *)c->d_sumbuf;
+    cudaError_t e = cudaSuccess;
+    for (uint32_t a = i; a < end && e == cudaSuccess;) {
+        const uint32_t z = sp_list_end(c, a, end);
+        SecondPassRange r{};
+        r.vlo = c->part_vb[a];
+        r.vhi = c->part_vb[z];
+        r.E0 = c->part_eb[a];
+        r.E1 = c->part_eb[z];
+        // a slice of the tile index: one spare tile per partition keeps the
+        // slices of neighbouring ranges apart
+        r.tbase = r.E0 / kTile + a;
+        r.cursor = c->d_sp_cursor + a;
+        r.edges_out = ctr;
+        r.dst = dst;
+        r.w = w;
+        r.shift = shift;
+        r.src_len = src_len;
+        if (a != i) e = launch_zero_u64(r.cursor, 1, s);
+        if (e != cudaSuccess) break;
+        if (c->batch_mode == kBatchPPR) {
+            BatchState b = c->bs;
+            b.loop = st.loop;
+            e = launch_second_pass_batched(b, c->d_off, r, la, sum, c->batch_K, (float)c->pr_damping,
+                                           (float)c->pr_eps, st.bm_cur, s);
+        } else {
+            e = launch_second_pass(st, c->d_off, r, la, sum, s);
+        }
+        a = z;
+    }
+    return e;
 }
 
 // An F task's range gets its second pass only if it holds at least
@@ -1101,6 +1172,7 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
         RelaxTask tc{}, tz{};
         tc.route = kRouteCache; tc.mode = kModeDevice; tc.dst = c->carve.cache_dst; tc.w = c->carve.cache_w;
         tc.shift = 0; tc.device_sized = true; tc.src_len = c->carve.cache_edges;
+        if (cache_second_pass_on(c, algo)) tc.sp_reset = sp_first_cursor(c, 0);
         tz.route = kRouteZ; tz.mode = kModeHost; tz.dst = c->m_dst; tz.w = c->m_w; tz.shift = 0;
         tz.device_sized = true; tz.src_len = c->E; tz.link_ctr = c->d_link_ctr + 2 * kRouteZ;
         {
@@ -1110,7 +1182,7 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
         if (cache_second_pass_on(c, algo)) {
             ScopedTime tm(c, kKindSecondPass, s);
             CK(second_pass_any(c, st, c->carve.cache_dst, c->carve.cache_w, 0, c->carve.cache_edges, 0,
-                               c->part_vb[c->carve.n_cached], 0, c->part_eb[c->carve.n_cached], c->d_sp, s));
+                               c->carve.n_cached, c->d_sp, s));
             count_second_launch(c);
         }
         return HYTG_OK;
@@ -1119,6 +1191,7 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
         RelaxTask t{};
         t.route = kRouteCache; t.mode = kModeDevice; t.dst = c->carve.cache_dst; t.w = c->carve.cache_w;
         t.shift = 0; t.device_sized = true; t.src_len = c->carve.cache_edges;
+        if (cache_second_pass_on(c, algo)) t.sp_reset = sp_first_cursor(c, 0);
         {
             ScopedTime tm(c, HYTG_K_RELAX_CACHE, s);
             CK(relax_any(c, st, la, sum, t, cap, s));
@@ -1128,7 +1201,7 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
             unsigned long long *ctr = next_sp_slot(c, &tm.sp_slot);
             tm.vertices = c->part_vb[c->carve.n_cached];
             CK(second_pass_any(c, st, c->carve.cache_dst, c->carve.cache_w, 0, c->carve.cache_edges, 0,
-                               c->part_vb[c->carve.n_cached], 0, c->part_eb[c->carve.n_cached], ctr, s));
+                               c->carve.n_cached, ctr, s));
             count_second_launch(c);
             c->stats.second_pass_vertices += c->part_vb[c->carve.n_cached];
         }
@@ -1229,15 +1302,17 @@ hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::ve
             t.route = kRouteF; t.mode = kModeDevice; t.dst = cv.slot_dst[L]; t.w = cv.slot_w[L];
             t.shift = (long long)e0; t.src_len = ee - e0;
             t.dev_edge = pa.route_edge + i; t.dev_len = pa.edges + i; t.dev_entry = pa.route_entry + i;
+            const bool again = second_pass_on(c, algo) &&
+                               range_second_pass(c, ee - eb, c->part_vb[i + 1] - c->part_vb[i]);
+            if (again) t.sp_reset = sp_first_cursor(c, i);
             if (e == cudaSuccess) {
                 ScopedTime tm(c, HYTG_K_RELAX_F, c->s_cap2);
                 e = relax_any(c, st, la, sum, t, cap, c->s_cap2);
             }
-            if (e == cudaSuccess && second_pass_on(c, algo) &&
-                range_second_pass(c, ee - eb, c->part_vb[i + 1] - c->part_vb[i])) {
+            if (e == cudaSuccess && again) {
                 ScopedTime tm(c, kKindSecondPass, c->s_cap2);
-                e = second_pass_any(c, st, cv.slot_dst[L], cv.slot_w[L], (long long)e0, ee - e0, c->part_vb[i],
-                                    c->part_vb[i + 1], eb, ee, c->d_sp, c->s_cap2);
+                e = second_pass_any(c, st, cv.slot_dst[L], cv.slot_w[L], (long long)e0, ee - e0, i, i + 1, c->d_sp,
+                                    c->s_cap2);
                 count_second_launch(c);
             }
         }
@@ -1719,6 +1794,8 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
         t.first_entry = p_rentry[i0];
         t.device_sized = false;
         t.src_len = e0 + edges - ea;
+        const bool again = second_pass_on(c, algo) && range_second_pass(c, edges, c->part_vb[j + 1] - c->part_vb[i0]);
+        if (again) t.sp_reset = sp_first_cursor(c, i0);
         {
             ScopedTime tm(c, HYTG_K_RELAX_F, fs);
             tm.edges = t.k_end - t.k_begin;
@@ -1726,14 +1803,14 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             tm.part_last = j;
             CK(relax_any(c, st, la, dsum, t, 8 * (int)device_sms(), fs));
         }
-        if (second_pass_on(c, algo) && range_second_pass(c, edges, c->part_vb[j + 1] - c->part_vb[i0])) {
+        if (again) {
             ScopedTime tm(c, kKindSecondPass, fs);
             unsigned long long *ctr = next_sp_slot(c, &tm.sp_slot);
             tm.vertices = c->part_vb[j + 1] - c->part_vb[i0];
             tm.part_first = i0;
             tm.part_last = j;
-            CK(second_pass_any(c, st, cv.slot_dst[slot], cv.slot_w[slot], (long long)ea, e0 + edges - ea,
-                               c->part_vb[i0], c->part_vb[j + 1], e0, c->part_eb[j + 1], ctr, fs));
+            CK(second_pass_any(c, st, cv.slot_dst[slot], cv.slot_w[slot], (long long)ea, e0 + edges - ea, i0, j + 1,
+                               ctr, fs));
             count_second_launch(c);
             c->stats.second_pass_vertices += c->part_vb[j + 1] - c->part_vb[i0];
         }
@@ -2151,8 +2228,6 @@ hytg_status hytg_load_csr(hytg_ctx *c, uint64_t V, uint64_t E, const uint64_t *o
         CK(cudaMalloc(&c->d_val, V * 4));
         CK(cudaMalloc(&c->d_delta, V * 4));
         CK(cudaMalloc(&c->d_out, V * 4));
-        CK(cudaMalloc(&c->d_sp_owner, (E / kSpChunk + 2) * 4));
-        CK(cudaMalloc(&c->d_sp_mask, c->n_words_alloc * 4));
         CK(cudaMalloc(&c->d_bm[0], c->n_words_alloc * 4));
         CK(cudaMemset(c->d_bm[0], 0, c->n_words_alloc * 4));
         CK(cudaMalloc(&c->d_ebase, V * 8));
@@ -2164,7 +2239,7 @@ hytg_status hytg_load_csr(hytg_ctx *c, uint64_t V, uint64_t E, const uint64_t *o
         hytg_status s = upload_partitions(c);
         if (s != HYTG_OK) return s;
         c->vertex_bytes = (V + 1) * 8 + 3 * V * 4 + c->n_words_alloc * 4 + V * 20 + n_tiles * 4 +
-                          c->sum_dev_bytes + (E / kSpChunk + 2) * 4 + c->n_words_alloc * 4;
+                          c->sum_dev_bytes;
         if (c->weighted) {
             // automatic SSSP bucket width: 8 x the mean edge weight (delta-stepping)
             long double sw = 0;
@@ -2357,6 +2432,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         hytg_status s = plan_carve(c, n_arrays);
         if (s != HYTG_OK) return s;
         s = ensure_cache(c, n_arrays);
+        if (s == HYTG_OK) s = ensure_second_pass(c, algo);
         if (s != HYTG_OK) return s;
         // delta-stepping bucket (SSSP only): eligible vertices have dist < bucket
         uint64_t delta = 0;
@@ -2655,6 +2731,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     c->serve_frames_used = 0;
     for (auto &f : c->serve_group_frame) f = -1;
     s = ensure_cache(c, n_arrays);
+    if (s == HYTG_OK) s = ensure_second_pass(c, algo);
     if (s != HYTG_OK) return s;
     CK(cudaMemsetAsync(c->d_err, 0, 4, c->s_main));
     CK(cudaMemsetAsync(c->d_overflow, 0, 4, c->s_main));
