@@ -464,10 +464,8 @@ const char *hytg_last_error(hytg_ctx *ctx);
  * memory, or a service that must not change its device footprint once it has
  * started.  hytg_plan_noalloc gives them the per-partition counting and
  * engine selection of hytg_plan (Sec. V-A, Eq. 1-3) without any allocation:
- * no context, no cudaMalloc/cudaFree and no allocating library call.  Its only
- * scratch is a static device array of HYTG_NOALLOC_MAX_PARTS + 1 partition
- * bounds (about 768 KiB), which every GPU that loads the library holds until
- * the process exits.
+ * no context, no cudaMalloc/cudaFree, no allocating library call and no scratch
+ * of its own: it reads the inputs and writes the two outputs.
  *
  * All pointers are device pointers owned by the caller:
  *   frontier      ceil(V / 32) uint32 words, bit v % 32 of word v / 32 set
@@ -484,14 +482,11 @@ const char *hytg_last_error(hytg_ctx *ctx);
  * stream is a cudaStream_t (NULL: the default stream); the work is queued on
  * it and the call returns without waiting.
  *
- * The first call on a device looks up the static array's device address
- * (cudaGetSymbolAddress) with that device current; make that first call
- * before any stream capture.  Every call shares the one array, so calls that
- * overlap on the GPU (on different streams, or from several threads) race:
- * order them on one stream.  Errors: HYTG_ERR_ARG for a NULL pointer, an
+ * Calls on different streams, or from several threads, may overlap as long as
+ * their outputs differ.  Errors: HYTG_ERR_ARG for a NULL pointer, an
  * unknown algorithm, V outside [1, 2^32 - 1], n_parts of 0 or above
  * HYTG_NOALLOC_MAX_PARTS, n_cached > n_parts or bad params; HYTG_ERR_CUDA if
- * the address lookup or a launch fails, or if a CUDA error left by earlier
+ * a launch fails, or if a CUDA error left by earlier
  * work is already pending when the call starts (nothing is queued then, and
  * that error is left pending for its owner to read). */
 #define HYTG_NOALLOC_MAX_PARTS 65536u
