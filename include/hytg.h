@@ -77,8 +77,9 @@ typedef struct hytg_stats {
     uint64_t route_partitions[5];     /* partition-iterations per route */
     uint64_t route_vertices[5];       /* active vertices (degree > 0) per route */
     uint64_t route_edges[5];          /* active edges per route */
-    uint64_t link_bytes[5];           /* host-link bytes per route: F whole partitions,
-                                         C and Z 128-byte lines spanned (C with
+    uint64_t link_bytes[5];           /* host-link bytes per route: F whole partitions as
+                                         copied (bit-packed, see hytg_load_csr),
+                                         C and Z the cost model's 128-byte lines (C with
                                          "compact_host": the active edge bytes plus 16 B of
                                          list index per vertex), cache 0 */
     uint64_t cache_fill_bytes;        /* bytes copied to fill the resident cache this run */
@@ -167,7 +168,9 @@ hytg_status hytg_destroy(hytg_ctx *ctx);
  * neighbour and weight arrays in host memory).  offsets: V+1 uint64, with
  * offsets[0] = 0, offsets[V] = E, non-decreasing; dst: E uint32, each < V;
  * weights: E uint32 or NULL for an unweighted graph.  The arrays are copied
- * into library-owned pinned, device-mapped host memory; the caller keeps
+ * into library-owned pinned, device-mapped host memory, bit-packed: a target
+ * takes ceil(log2 V) bits and a weight the bits of the largest weight (the
+ * cost model of Sec. V-A keeps 4 bytes per entry); the caller keeps
  * ownership of its arrays.  V must be in [1, 2^32 - 1].  Replaces any earlier
  * graph.  Errors: HYTG_ERR_ARG (bad CSR), HYTG_ERR_HOSTMEM, HYTG_ERR_CUDA. */
 hytg_status hytg_load_csr(hytg_ctx *ctx, uint64_t V, uint64_t E, const uint64_t *offsets,
@@ -204,10 +207,9 @@ hytg_status hytg_set_device_budget(hytg_ctx *ctx, uint64_t bytes);
  * from its slot, in its place in the order; counted in f_ahead_tasks /
  * f_ahead_hits; when on, "slot_reuse" is not applied; 0: off),
  * "f_copy" (0, default: F copies by the copy engine, cudaMemcpyAsync; n in
- * 1..32: by a kernel with n blocks per SM that reads the task's edges from
- * mapped host memory with 16-byte loads, starting at the 16-byte boundary
- * at or below the first edge when the slot has room for the up to 3 extra
- * words read, else by the copy engine),
+ * 1..32: by a kernel with n blocks per SM that reads the task's words from
+ * mapped host memory with 16-byte loads; either way a copy starts at the
+ * 16-byte boundary at or below the task's first edge),
  * "timing" (1: CUDA-event time per kernel
  * kind), "hub_frac" (fraction of vertices moved to the front by hub sorting
  * at the next hytg_load_csr, Sec. VI-A; 0 disables it; default 0.08),

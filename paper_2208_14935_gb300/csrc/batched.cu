@@ -214,8 +214,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
     walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
         unsigned int dv[kBatchSteps];
         unsigned long long vis[kBatchSteps];
-#pragma unroll
-        for (int q = 0; q < kBatchSteps; ++q) dv[q] = ed[q].ok ? __ldg(t.dst + ed[q].e) : 0u;
+        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
 #pragma unroll
         for (int q = 0; q < kBatchSteps; ++q) vis[q] = ed[q].ok ? __ldcg(&b.vis[dv[q]]) : ~0ull;
 #pragma unroll
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
             if (ed[q].ok && nb) atomicOr(&b.nxt[dv[q]], nb);
         }
     });
-    flush_link(lc, 1u, t.link_ctr);
+    flush_link(lc, t.link_ctr);
 }
 
 // Multi-source SSSP and batched PPR relax.  A warp loads 32 edges at once
@@ -294,16 +293,11 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, List
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     LinkCount lc;
+    lc.weights = MODE == kBatchSSSP;
     walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
-        unsigned int dv[kBatchSteps], wv[kBatchSteps];
-#pragma unroll
-        for (int q = 0; q < kBatchSteps; ++q) {
-            dv[q] = wv[q] = 0;
-            if (ed[q].ok) {
-                dv[q] = __ldg(t.dst + ed[q].e);
-                if (MODE == kBatchSSSP) wv[q] = __ldg(t.w + ed[q].e);
-            }
-        }
+        unsigned int dv[kBatchSteps], wv[kBatchSteps] = {};
+        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
+        if (MODE == kBatchSSSP) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
 #pragma unroll
         for (int q = 0; q < kBatchSteps; ++q) {
             const unsigned long long f = ed[q].ok ? ed[q].pay : 0ull;
@@ -318,7 +312,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, List
             }
         }
     });
-    flush_link(lc, MODE == kBatchSSSP ? 2u : 1u, t.link_ctr);
+    flush_link(lc, t.link_ctr);
 }
 
 // Batched PPR second pass over a resident range [vlo, vhi) (Sec. VI-A): the

@@ -258,16 +258,32 @@ cudaError_t launch_bin(const GraphDev &g, const AlgoState &st, const PartArrays 
 // Edge source of a relax / gather launch.
 enum EdgeMode : int { kModeHost = 0, kModeDevice = 1, kModeCompact = 2 };
 
+// The edge arrays a task reads, in host memory or copied to the device.  The
+// CSR arrays are bit-packed at load: entry e takes `bits` bits, from bit
+// e * bits - off of the array (least significant bit first), so any run of
+// edges is a run of words that can be copied or read as it is.  Targets take
+// ceil(log2 V) bits and weights those of the largest one: on R-MAT 24 with
+// weights up to 64, 24 and 7 bits of 32 each, so the host link, the staging
+// slots and the cache move or hold 1.3x (BFS, CC, PageRank) to 2.1x (SSSP)
+// more edges per byte.  Such runs are bound by the link: at a budget of 25 %
+// of the graph (R-MAT 24, device time) BFS went from 6.0 to 3.9 ms, SSSP from
+// 22.8 to 10.7 ms, PPR from 278 to 229 ms (46 -> 24 GB copied).  Entries keep
+// a fixed width rather than gaps of sorted rows, so any edge of any row order
+// is found by its index alone.  The compaction buffer holds plain words.
+struct EdgeSrc {
+    const unsigned int *dst, *w;        // targets; weights or nullptr
+    unsigned int dst_bits, w_bits;
+    long long dst_off, w_off;
+    unsigned long long e_lo, e_hi;      // edges present: [e_lo, e_hi)
+};
+
 struct RelaxTask {
     int route;                          // which route's list / tiles
-    int mode;                           // EdgeMode
-    const unsigned int *dst;            // edge destinations (device or mapped host)
-    const unsigned int *w;              // weights or nullptr
-    long long shift;                    // edge index of dst[0] (device copies)
+    int mode;                           // EdgeMode: in a compacted buffer an edge is its place in the route
+    EdgeSrc src;
     unsigned long long k_begin, k_end;  // edge range in the route's edge space
     unsigned long long first_entry;     // route-relative entry holding k_begin
     bool device_sized;                  // take k_end from the summary (k_begin = 0)
-    unsigned long long src_len;         // valid indices of dst / w: [0, src_len)
     unsigned long long *link_ctr;       // host-memory reads (Z relax, C gather): {32-byte
                                         // sectors, 128-byte lines} read, or nullptr
     // One partition's F task inside the device loop: its first edge in the F
@@ -291,7 +307,7 @@ cudaError_t launch_relax(const AlgoState &st, const ListArrays &la, const Summar
 cudaError_t launch_relax_pair(const AlgoState &st, const ListArrays &la, const Summary *sum,
                               const RelaxTask &ta, const RelaxTask &tb, int grid, cudaStream_t s);
 // Second pass (Sec. VI-A) over vertices [vlo, vhi) (vlo a multiple of 32)
-// whose edges [E0, E1) are resident in dst / w (CSR edge shift at index 0):
+// whose edges [E0, E1) are resident in src:
 // a take launch, which lists the vertices it takes as k_bin lists a route's,
 // and a relax over that list.  The list's entries lie at [vlo, vhi) and its
 // tiles from `tbase` of arrays shared by every second pass of a run, whose
@@ -301,9 +317,7 @@ struct SecondPassRange {
     unsigned long long tbase;            // first tile of the range's slice
     unsigned long long *cursor;          // packed entries and edges of its list
     unsigned long long *edges_out;       // statistics: edges taken
-    const unsigned int *dst, *w;
-    long long shift;
-    unsigned long long src_len;
+    EdgeSrc src;
 };
 cudaError_t launch_second_pass(const AlgoState &st, const unsigned long long *off, const SecondPassRange &r,
                                const ListArrays &la, const Summary *sum, cudaStream_t s);

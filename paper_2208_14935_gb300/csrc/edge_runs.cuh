@@ -74,38 +74,72 @@ __device__ __forceinline__ RouteView task_view(RelaxTask &t, const Summary *sum,
     return rv;
 }
 
-// Host-link reads of a task that reads mapped host memory: the distinct
-// 32-byte sectors and 128-byte lines that its edges occupy in one 4-byte edge
-// array (base 256-byte aligned, so edge e sits in sector e / 8 and line
-// e / 32).  The edges of an entry are at increasing addresses, so a sector
-// (line) is new where it differs from the previous edge's; a run's first edge
-// is compared with the edge before it.  Per-lane counts, added once per warp.
+// Host-link reads of a task that reads mapped host memory: the 32-byte sectors
+// and 128-byte lines that its edges' entries occupy in each array read (base
+// 256-byte aligned).  The edges of an entry are at increasing addresses, so a
+// sector (line) is new where it differs from the one the previous edge ended
+// in; a run's first edge is compared with the edge before it.  Per-lane
+// counts, added once per warp.
 struct LinkCount {
     unsigned int sec = 0, ln = 0;
+    bool weights = false;               // the weight array is read too
 };
-__device__ __forceinline__ void flush_link(const LinkCount &lc, unsigned int n_arrays, unsigned long long *ctr) {
+__device__ __forceinline__ void count_link(LinkCount &lc, long long e, long long prev, unsigned int bits) {
+    const unsigned long long a = (unsigned long long)e * bits, z = a + bits - 1;
+    const unsigned long long p = prev < 0 ? ~0ull : (unsigned long long)prev * bits + bits - 1;
+    lc.sec += ((a >> 8) != (p >> 8)) + ((z >> 8) != (a >> 8));
+    lc.ln += ((a >> 10) != (p >> 10)) + ((z >> 10) != (a >> 10));
+}
+__device__ __forceinline__ void flush_link(const LinkCount &lc, unsigned long long *ctr) {
     if (!ctr) return;
     const unsigned int sec = __reduce_add_sync(0xffffffffu, lc.sec), ln = __reduce_add_sync(0xffffffffu, lc.ln);
     if ((threadIdx.x & 31) == 0 && sec) {
-        atomicAdd(&ctr[0], (unsigned long long)sec * n_arrays);
-        atomicAdd(&ctr[1], (unsigned long long)ln * n_arrays);
+        atomicAdd(&ctr[0], (unsigned long long)sec);
+        atomicAdd(&ctr[1], (unsigned long long)ln);
     }
 }
 
-// One edge of a step: its index in the task's edge arrays and its owner's
+// One edge of a step: its CSR index (compacted buffer: its place in the
+// route), whether the next lane holds the edge after it, and its owner's
 // payload.  BATCH: the owner's per-source word and vertex instead of a value.
 template <bool BATCH> struct Edge;
 template <> struct Edge<false> {
-    bool ok;
+    bool ok, adj;
     long long e;
     unsigned int pay;
 };
 template <> struct Edge<true> {
-    bool ok;
+    bool ok, adj;
     long long e;
     unsigned long long pay;
     unsigned int vid;
 };
+
+// The packed entries of a lane's S edges (0 where there is none).  An entry
+// that runs into the next word takes that word from the next lane when that
+// lane holds the next edge (its entry then starts in that word), so a list's
+// words are loaded once; only a list's or a step's last edge may load a second
+// word.  Needs all 32 lanes.
+template <int S, class E>
+__device__ __forceinline__ void load_entries(const unsigned int *p, unsigned int bits, long long off,
+                                             const E (&ed)[S], unsigned int (&out)[S]) {
+    const unsigned int mask = 0xffffffffu >> (32 - bits);
+    unsigned int lo[S], sh[S];
+    long long at[S];
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        const long long bit = ed[q].ok ? ed[q].e * (long long)bits - off : 0;
+        at[q] = bit >> 5;
+        sh[q] = (unsigned int)bit & 31u;
+        lo[q] = ed[q].ok ? __ldg(p + at[q]) : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        unsigned int hi = __shfl_down_sync(0xffffffffu, lo[q], 1);
+        if (ed[q].ok && !ed[q].adj && sh[q] + bits > 32) hi = __ldg(p + at[q] + 1);
+        out[q] = ed[q].ok ? __funnelshift_r(lo[q], hi, sh[q]) & mask : 0u;
+    }
+}
 
 // Run length (log2) for `total` edges over `nwarps` warps: kRun, halved down
 // to one step of 32 edges while there are fewer runs than warps, so that a
@@ -162,7 +196,7 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
             const long long eb = (long long)la.ebase[idx];
             const long long d = eb - (long long)k0;
             rel = d < 0 ? -1 : d < (long long)kRun ? (int)d : kRun;
-            delta = t.mode == kModeCompact ? -t.shift : (long long)la.soff[idx] - eb - t.shift;
+            delta = t.mode == kModeCompact ? 0 : (long long)la.soff[idx] - eb;
             if (BATCH) {
                 pay64 = la.pay64[idx];
                 vid = la.vid[idx];
@@ -188,7 +222,7 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
                 e_prev = (long long)(k0 - 1) + __shfl_sync(0xffffffffu, delta, 31 - __clz(le));
             } else {                                // k0 starts the window's first list
                 const unsigned long long j = rv.rbase + (i ? i - 1 : 0);
-                e_prev = (long long)(k0 - 1) + ((long long)la.soff[j] - (long long)la.ebase[j] - t.shift);
+                e_prev = (long long)(k0 - 1) + ((long long)la.soff[j] - (long long)la.ebase[j]);
             }
         }
         for (int b0 = pos; b0 < wend; b0 += 32 * S) {
@@ -196,7 +230,7 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
 #pragma unroll
             for (int q = 0; q < S; ++q) {
                 const int b = b0 + 32 * q;
-                ed[q].ok = false;
+                ed[q].ok = ed[q].adj = false;
                 if (b >= wend) continue;            // warp-uniform
                 const int before = __popc(__ballot_sync(0xffffffffu, rel < b));
                 const unsigned int heads =
@@ -210,18 +244,19 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
                     ed[q].pay = __shfl_sync(0xffffffffu, pay, own);
                 }
                 ed[q].ok = b + lane < wend;
+                ed[q].adj = lane < 31 && b + lane + 1 < wend && !((heads >> (lane + 1)) & 1u);
                 if (t.link_ctr) {
                     long long p = __shfl_up_sync(0xffffffffu, ed[q].e, 1);
                     if (lane == 0) p = e_prev;
                     if (ed[q].ok) {
-                        lc.sec += (ed[q].e >> 3) != (p >> 3);
-                        lc.ln += (ed[q].e >> 5) != (p >> 5);
+                        count_link(lc, ed[q].e, p, t.src.dst_bits);
+                        if (lc.weights) count_link(lc, ed[q].e, p, t.src.w_bits);
                     }
                     e_prev = __shfl_sync(0xffffffffu, ed[q].e, min(31, wend - 1 - b));
                 }
-                if (ed[q].ok && (ed[q].e < 0 || (unsigned long long)ed[q].e >= t.src_len)) {
+                if (ed[q].ok && (ed[q].e < (long long)t.src.e_lo || ed[q].e >= (long long)t.src.e_hi)) {
                     atomicOr(la.err, 8u);
-                    ed[q].ok = false;
+                    ed[q].ok = ed[q].adj = false;
                 }
             }
             f(ed, k0 + b0 + lane);
@@ -283,10 +318,7 @@ inline unsigned int run_blocks(unsigned long long kb, unsigned long long ke, uns
 inline RelaxTask sp_push_task(const SecondPassRange &r) {
     RelaxTask t{};
     t.mode = kModeDevice;
-    t.dst = r.dst;
-    t.w = r.w;
-    t.shift = r.shift;
-    t.src_len = r.src_len;
+    t.src = r.src;
     t.device_sized = true;
     t.sp_cursor = r.cursor;
     t.sp_rbase = r.vlo;

@@ -152,7 +152,8 @@ struct hytg_ctx {
     int symmetric = -1;                                  // CSR symmetry: -1 not checked yet, 0 no, 1 yes
     uint64_t V = 0, E = 0;
     bool weighted = false;
-    uint32_t *h_dst = nullptr, *h_w = nullptr;          // pinned, mapped
+    uint32_t *h_dst = nullptr, *h_w = nullptr;          // pinned, mapped, bit-packed (EdgeSrc)
+    unsigned int dst_bits = 32, w_bits = 32;             // bits per target and per weight
     size_t h_map_bytes[2] = {};                          // "host_huge": mmap'd length of h_dst / h_w (0: cudaHostAlloc)
     void *h_map_base[2] = {};
     const uint32_t *m_dst = nullptr, *m_w = nullptr;    // device view of the same memory
@@ -360,7 +361,60 @@ void free_loop_graph(hytg_ctx *c) {
     c->loop_key.clear();
 }
 
-void parallel_chunks(uint64_t n, const std::function<void(uint64_t, uint64_t)> &fn);
+void parallel_chunks(uint64_t n, const std::function<void(uint64_t, uint64_t)> &fn, uint64_t serial = 1u << 20);
+
+// ---- bit-packed edge arrays (see EdgeSrc)
+unsigned int bits_for(uint64_t max_value) {
+    unsigned int b = 1;
+    while (b < 32 && (max_value >> b) != 0) ++b;
+    return b;
+}
+
+// Words that hold n entries from a word boundary, with a word to spare (an
+// entry's second word) and rounded to 16 bytes.
+uint64_t packed_words(uint64_t n, unsigned int bits) { return ((n * bits + 31) / 32 + 1 + 3) & ~uint64_t(3); }
+
+// The words to copy for entries [e0, e0 + n): from the 16-byte boundary at or
+// below the first entry to the word of the last one.
+struct WordSpan {
+    uint64_t w0, n;
+};
+WordSpan word_span(uint64_t e0, uint64_t n, unsigned int bits) {
+    const uint64_t w0 = (e0 * bits / 32) & ~uint64_t(3);
+    return {w0, n ? ((e0 + n) * bits + 31) / 32 - w0 : 0};
+}
+
+inline uint32_t packed_get(const uint32_t *a, unsigned int bits, uint64_t e) {
+    const uint64_t bit = e * bits;
+    const unsigned int sh = (unsigned int)(bit & 31);
+    uint64_t x = a[bit >> 5];
+    if (sh + bits > 32) x |= (uint64_t)a[(bit >> 5) + 1] << 32;
+    return (uint32_t)((x >> sh) & (0xFFFFFFFFull >> (32 - bits)));
+}
+
+// Writes consecutive entries from entry `e`, a multiple of 32 (a word
+// boundary whatever the width); finish() writes the last, partial word.
+class PackedWriter {
+public:
+    PackedWriter(uint32_t *a, unsigned int bits, uint64_t e) : p_(a + e * bits / 32), bits_(bits) {}
+    void put(uint32_t v) {
+        acc_ |= (uint64_t)v << fill_;
+        fill_ += bits_;
+        if (fill_ >= 32) {
+            *p_++ = (uint32_t)acc_;
+            acc_ >>= 32;
+            fill_ -= 32;
+        }
+    }
+    void finish() {
+        if (fill_) *p_++ = (uint32_t)acc_;
+    }
+
+private:
+    uint32_t *p_;
+    unsigned int bits_, fill_ = 0;
+    uint64_t acc_ = 0;
+};
 
 hytg_status alloc_edge_array_huge(hytg_ctx *c, int a, uint32_t **out, size_t bytes);
 
@@ -455,9 +509,11 @@ void free_graph(hytg_ctx *c) {
     c->carve = Carve();
 }
 
-void parallel_chunks(uint64_t n, const std::function<void(uint64_t, uint64_t)> &fn) {
+// fn over [0, n) in one piece per host thread; fewer than `serial` items stay
+// on the calling thread.
+void parallel_chunks(uint64_t n, const std::function<void(uint64_t, uint64_t)> &fn, uint64_t serial) {
     unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-    if (n < (1u << 20)) nt = 1;
+    if (n < serial) nt = 1;
     std::vector<std::thread> th;
     for (unsigned t = 1; t < nt; ++t) th.emplace_back(fn, n * t / nt, n * (t + 1) / nt);
     fn(0, n / nt);
@@ -489,11 +545,12 @@ void parallel_edge_balanced(const std::vector<uint64_t> &off, uint64_t V,
 // reverse.  In-degrees must equal out-degrees; the reverse rows then have the
 // CSR's own offsets, and each row, sorted, must equal the sorted list of the
 // vertex's in-neighbours.  O(E) plus the row sorts, on host threads.
-bool csr_symmetric(const std::vector<uint64_t> &off, const uint32_t *dst, uint64_t V) {
+bool csr_symmetric(const std::vector<uint64_t> &off, const uint32_t *packed, unsigned int bits, uint64_t V) {
     const uint64_t E = off[V];
+    const auto dst = [&](uint64_t e) { return packed_get(packed, bits, e); };
     std::vector<uint64_t> indeg(V, 0);
     parallel_chunks(E, [&](uint64_t lo, uint64_t hi) {
-        for (uint64_t e = lo; e < hi; ++e) __atomic_fetch_add(&indeg[dst[e]], 1ull, __ATOMIC_RELAXED);
+        for (uint64_t e = lo; e < hi; ++e) __atomic_fetch_add(&indeg[dst(e)], 1ull, __ATOMIC_RELAXED);
     });
     std::atomic<bool> ok{true};
     parallel_chunks(V, [&](uint64_t lo, uint64_t hi) {
@@ -506,14 +563,15 @@ bool csr_symmetric(const std::vector<uint64_t> &off, const uint32_t *dst, uint64
     parallel_edge_balanced(off, V, [&](uint64_t lo, uint64_t hi) {
         for (uint64_t u = lo; u < hi; ++u)
             for (uint64_t e = off[u]; e < off[u + 1]; ++e)
-                rev[__atomic_fetch_add(&cur[dst[e]], 1ull, __ATOMIC_RELAXED)] = (uint32_t)u;
+                rev[__atomic_fetch_add(&cur[dst(e)], 1ull, __ATOMIC_RELAXED)] = (uint32_t)u;
     });
     parallel_edge_balanced(off, V, [&](uint64_t lo, uint64_t hi) {
         std::vector<uint32_t> row;
         for (uint64_t v = lo; v < hi && ok; ++v) {
             const uint64_t b = off[v], n = off[v + 1] - b;
             if (n == 0) continue;
-            row.assign(dst + b, dst + b + n);
+            row.resize(n);
+            for (uint64_t j = 0; j < n; ++j) row[j] = dst(b + j);
             std::sort(row.begin(), row.end());
             std::sort(rev.begin() + b, rev.begin() + b + n);
             if (!std::equal(row.begin(), row.end(), rev.begin() + b)) ok = false;
@@ -667,23 +725,33 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
                                             " B is below one staging slot of the largest partition (" +
                                             std::to_string(min_slot * eb) + " B) plus the minimum compaction buffer (" +
                                             std::to_string(compact_min * eb) + " B)");
+    // sizes are those of the packed arrays; the refusal above is by plain
+    // 4-byte entries, which are never smaller
+    auto bytes = [&](uint64_t edges) {
+        return 4 * (packed_words(edges, c->dst_bits) + (n_arrays == 2 ? packed_words(edges, c->w_bits) : 0));
+    };
+    const uint64_t slack = 64;                     // alignment of a slot's first entry, spare words
     uint64_t stage_cap = std::max<uint64_t>((uint64_t)(B * c->staging_frac), min_slot * eb);
     stage_cap = std::min<uint64_t>(stage_cap, B - compact_min * eb);
     uint64_t slot_edges = std::max<uint64_t>((uint64_t)c->k * pe, min_slot);
-    if (slot_edges * eb > stage_cap) slot_edges = std::max<uint64_t>(min_slot, stage_cap / eb);
-    uint64_t n_slots = stage_cap / (slot_edges * eb);
+    if (bytes(slot_edges) > stage_cap) {
+        const unsigned int ebits = c->dst_bits + (n_arrays == 2 ? c->w_bits : 0);
+        slot_edges = std::max<uint64_t>(min_slot, stage_cap > slack ? (stage_cap - slack) * 8 / ebits : 0);
+    }
+    uint64_t n_slots = stage_cap / std::max<uint64_t>(1, bytes(slot_edges));
     n_slots = std::max<uint64_t>(1, std::min<uint64_t>({n_slots, (uint64_t)(c->streams + c->prefetch_slots),
                                                         (uint64_t)kMaxSlots}));
-    uint64_t rem = B - n_slots * slot_edges * eb;
+    const uint64_t staged = n_slots * bytes(slot_edges);
+    uint64_t rem = B > staged ? B - staged : 0;
     uint64_t compact_edges = std::max<uint64_t>(compact_min, (uint64_t)(B * c->compact_frac) / eb);
     compact_edges = std::min<uint64_t>(compact_edges, rem / eb);
     compact_edges = compact_edges / kCompactUnit * kCompactUnit;
     if (compact_edges < (uint64_t)kCompactUnit) compact_edges = kCompactUnit;
-    rem -= compact_edges * eb;
+    rem = rem > compact_edges * eb ? rem - compact_edges * eb : 0;
     // cache: largest prefix of whole partitions that fits
     uint32_t n_cached = 0;
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
-    while (n_cached < N && c->part_eb[n_cached + 1] * eb <= rem) ++n_cached;
+    while (n_cached < N && bytes(c->part_eb[n_cached + 1]) <= rem) ++n_cached;
     n.slot_edges = slot_edges;
     n.n_slots = (uint32_t)n_slots;
     n.compact_edges = compact_edges;
@@ -693,19 +761,27 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     auto align = [](uint64_t x) { return (x + 255) & ~uint64_t(255); };
     char *base = (char *)c->d_pool;
     uint64_t o = 0;
-    n.cache_dst = (uint32_t *)(base + o); o = align(o + n.cache_edges * 4);
-    if (n_arrays == 2) { n.cache_w = (uint32_t *)(base + o); o = align(o + n.cache_edges * 4); }
+    auto piece = [&](uint64_t nbytes) {
+        uint32_t *p = (uint32_t *)(base + o);
+        o = align(o + nbytes);
+        return p;
+    };
+    // a slot's first entry may lie up to 3 words and 31 bits into it
+    const uint64_t slot_d = 4 * packed_words(slot_edges, c->dst_bits) + 16;
+    const uint64_t slot_w = 4 * packed_words(slot_edges, c->w_bits) + 16;
+    n.cache_dst = piece(4 * packed_words(n.cache_edges, c->dst_bits));
+    if (n_arrays == 2) n.cache_w = piece(4 * packed_words(n.cache_edges, c->w_bits));
     for (uint32_t s = 0; s < n.n_slots; ++s) {
-        n.slot_dst[s] = (uint32_t *)(base + o); o = align(o + slot_edges * 4);
-        if (n_arrays == 2) { n.slot_w[s] = (uint32_t *)(base + o); o = align(o + slot_edges * 4); }
+        n.slot_dst[s] = piece(slot_d);
+        if (n_arrays == 2) n.slot_w[s] = piece(slot_w);
     }
-    n.cmp_dst = (uint32_t *)(base + o); o = align(o + compact_edges * 4);
-    if (n_arrays == 2) { n.cmp_w = (uint32_t *)(base + o); o = align(o + compact_edges * 4); }
+    n.cmp_dst = piece(compact_edges * 4);
+    if (n_arrays == 2) n.cmp_w = piece(compact_edges * 4);
     // at most 36 pieces, each padded by < 256 B: the pool holds budget + kPoolSlack
     if (o > B + kPoolSlack)
         return fail(c, HYTG_ERR_BUDGET, "internal: budget carve exceeds the pool");
     n.end = o;
-    n.used = n.cache_edges * eb + n.n_slots * slot_edges * eb + compact_edges * eb;
+    n.used = bytes(n.cache_edges) + n.n_slots * bytes(slot_edges) + compact_edges * eb;
     if (c->cache_filled_arrays != n_arrays || c->carve.cache_dst != n.cache_dst ||
         c->cache_filled_n != n.n_cached)
         c->cache_filled_arrays = 0;   // cache must be refilled
@@ -715,6 +791,41 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     if (!same_slots) slots_forget(c);
     cv = n;
     return HYTG_OK;
+}
+
+// The edge sources of tasks: the host arrays, the cache, a staging slot that
+// holds edges [e0, e0 + n), the compaction buffer with route edges [cb, ce).
+EdgeSrc edges_at(const hytg_ctx *c, const uint32_t *dst, const uint32_t *w, uint64_t e_lo, uint64_t e_hi) {
+    EdgeSrc x;
+    x.dst = dst;
+    x.w = w;
+    x.dst_bits = c->dst_bits;
+    x.w_bits = c->w_bits;
+    x.dst_off = x.w_off = 0;
+    x.e_lo = e_lo;
+    x.e_hi = e_hi;
+    return x;
+}
+EdgeSrc host_edges(const hytg_ctx *c) { return edges_at(c, c->m_dst, c->m_w, 0, c->E); }
+EdgeSrc cache_edges(const hytg_ctx *c) {
+    return edges_at(c, c->carve.cache_dst, c->carve.cache_w, 0, c->carve.cache_edges);
+}
+EdgeSrc slot_edges(const hytg_ctx *c, uint32_t slot, uint64_t e0, uint64_t n) {
+    EdgeSrc x = edges_at(c, c->carve.slot_dst[slot], c->carve.slot_w[slot], e0, e0 + n);
+    x.dst_off = (long long)word_span(e0, n, c->dst_bits).w0 * 32;
+    x.w_off = (long long)word_span(e0, n, c->w_bits).w0 * 32;
+    return x;
+}
+EdgeSrc compact_edges(const hytg_ctx *c, uint64_t cb, uint64_t ce) {
+    EdgeSrc x = edges_at(c, c->carve.cmp_dst, c->carve.cmp_w, cb, ce);
+    x.dst_bits = x.w_bits = 32;
+    x.dst_off = x.w_off = (long long)cb * 32;
+    return x;
+}
+
+// Bytes that a copy of edges [e0, e0 + n) moves.
+uint64_t copy_bytes(const hytg_ctx *c, uint64_t e0, uint64_t n, int n_arrays) {
+    return 4 * (word_span(e0, n, c->dst_bits).n + (n_arrays == 2 ? word_span(e0, n, c->w_bits).n : 0));
 }
 
 cudaEvent_t pool_event(hytg_ctx *c) {
@@ -960,8 +1071,7 @@ unsigned long long *sp_first_cursor(const hytg_ctx *c, uint32_t i) { return c->d
 
 // The second pass over the resident partitions [i, end), single-source or
 // batched PPR.
-cudaError_t second_pass_any(hytg_ctx *c, const AlgoState &st, const unsigned int *dst, const unsigned int *w,
-                            long long shift, unsigned long long src_len, uint32_t i, uint32_t end,
+cudaError_t second_pass_any(hytg_ctx *c, const AlgoState &st, const EdgeSrc &src, uint32_t i, uint32_t end,
                             unsigned long long *ctr, cudaStream_t s) {
     const ListArrays la = sp_list_arrays(c);
     const Summary *sum = (const Summary *)c->d_sumbuf;
@@ -978,10 +1088,7 @@ cudaError_t second_pass_any(hytg_ctx *c, const AlgoState &st, const unsigned int
         r.tbase = r.E0 / kTile + a;
         r.cursor = c->d_sp_cursor + a;
         r.edges_out = ctr;
-        r.dst = dst;
-        r.w = w;
-        r.shift = shift;
-        r.src_len = src_len;
+        r.src = src;
         if (a != i) e = launch_zero_u64(r.cursor, 1, s);
         if (e != cudaSuccess) break;
         if (c->batch_mode == kBatchPPR) {
@@ -1170,27 +1277,24 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
     if (c->capturing && c->batch_mode == kBatchNone && c->carve.n_cached > 0) {
         // device loop body: cache and zero-copy routes in one launch
         RelaxTask tc{}, tz{};
-        tc.route = kRouteCache; tc.mode = kModeDevice; tc.dst = c->carve.cache_dst; tc.w = c->carve.cache_w;
-        tc.shift = 0; tc.device_sized = true; tc.src_len = c->carve.cache_edges;
+        tc.route = kRouteCache; tc.mode = kModeDevice; tc.src = cache_edges(c); tc.device_sized = true;
         if (cache_second_pass_on(c, algo)) tc.sp_reset = sp_first_cursor(c, 0);
-        tz.route = kRouteZ; tz.mode = kModeHost; tz.dst = c->m_dst; tz.w = c->m_w; tz.shift = 0;
-        tz.device_sized = true; tz.src_len = c->E; tz.link_ctr = c->d_link_ctr + 2 * kRouteZ;
+        tz.route = kRouteZ; tz.mode = kModeHost; tz.src = host_edges(c); tz.device_sized = true;
+        tz.link_ctr = c->d_link_ctr + 2 * kRouteZ;
         {
             ScopedTime tm(c, HYTG_K_RELAX_Z, s);
             CK(launch_relax_pair(st, la, sum, tc, tz, cap, s));
         }
         if (cache_second_pass_on(c, algo)) {
             ScopedTime tm(c, kKindSecondPass, s);
-            CK(second_pass_any(c, st, c->carve.cache_dst, c->carve.cache_w, 0, c->carve.cache_edges, 0,
-                               c->carve.n_cached, c->d_sp, s));
+            CK(second_pass_any(c, st, cache_edges(c), 0, c->carve.n_cached, c->d_sp, s));
             count_second_launch(c);
         }
         return HYTG_OK;
     }
     if (c->carve.n_cached > 0) {
         RelaxTask t{};
-        t.route = kRouteCache; t.mode = kModeDevice; t.dst = c->carve.cache_dst; t.w = c->carve.cache_w;
-        t.shift = 0; t.device_sized = true; t.src_len = c->carve.cache_edges;
+        t.route = kRouteCache; t.mode = kModeDevice; t.src = cache_edges(c); t.device_sized = true;
         if (cache_second_pass_on(c, algo)) t.sp_reset = sp_first_cursor(c, 0);
         {
             ScopedTime tm(c, HYTG_K_RELAX_CACHE, s);
@@ -1200,16 +1304,15 @@ hytg_status issue_plan_tail(hytg_ctx *c, int algo, unsigned int bucket, cudaStre
             ScopedTime tm(c, kKindSecondPass, s);
             unsigned long long *ctr = next_sp_slot(c, &tm.sp_slot);
             tm.vertices = c->part_vb[c->carve.n_cached];
-            CK(second_pass_any(c, st, c->carve.cache_dst, c->carve.cache_w, 0, c->carve.cache_edges, 0,
-                               c->carve.n_cached, ctr, s));
+            CK(second_pass_any(c, st, cache_edges(c), 0, c->carve.n_cached, ctr, s));
             count_second_launch(c);
             c->stats.second_pass_vertices += c->part_vb[c->carve.n_cached];
         }
     }
     {
         RelaxTask t{};
-        t.route = kRouteZ; t.mode = kModeHost; t.dst = c->m_dst; t.w = c->m_w; t.shift = 0;
-        t.device_sized = true; t.src_len = c->E; t.link_ctr = c->d_link_ctr + 2 * kRouteZ;
+        t.route = kRouteZ; t.mode = kModeHost; t.src = host_edges(c); t.device_sized = true;
+        t.link_ctr = c->d_link_ctr + 2 * kRouteZ;
         ScopedTime tm(c, HYTG_K_RELAX_Z, s);
         CK(relax_any(c, st, la, sum, t, (int)c->z_blocks * (int)device_sms(), s));
     }
@@ -1226,14 +1329,12 @@ bool loop_applies(const hytg_ctx *c) {
 // F and C iterations can stay in the device loop: batched runs at "device_loop"
 // 1, every run at 2; not with host compaction, forced random routes, more
 // partitions than 1024 IF nodes, or a staging slot without room for one
-// partition (plus 3 words of alignment slack when the copy kernel, not a
-// memcpy node, moves it).
+// partition.
 bool loop_fc_wanted(const hytg_ctx *c) {
     if (c->device_loop < 2 && c->batch_mode == kBatchNone) return false;
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
-    const uint64_t slack = c->loop_fc_copy == 1 ? 3 : 0;
     return c->compact_host == 0 && c->force_route != 5 && N >= 1 && N <= 1024 && c->carve.n_slots >= 1 &&
-           c->carve.slot_edges >= c->max_part_edges + slack;
+           c->carve.slot_edges >= c->max_part_edges;
 }
 
 // One IF node per partition (copy the partition into the staging slot of its
@@ -1281,26 +1382,23 @@ hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::ve
         c->loop_fh[i] = (unsigned long long)h;
         lane[L] = node;
         const uint64_t eb = c->part_eb[i], ee = c->part_eb[i + 1];
-        // the copy kernel reads from the 16-byte boundary at or below the
-        // partition's first edge; a memcpy node copies the partition exactly
-        const uint64_t e0 = c->loop_fc_copy == 1 ? (eb & ~uint64_t(3)) : eb;
+        const WordSpan sd = word_span(eb, ee - eb, c->dst_bits), sw = word_span(eb, ee - eb, c->w_bits);
         CK(cudaStreamBeginCaptureToGraph(c->s_cap2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         hytg_status r = HYTG_OK;
         cudaError_t e = cudaSuccess;
         if (ee > eb) {
             if (c->loop_fc_copy == 0) {
-                e = cudaMemcpyAsync(cv.slot_dst[L], c->h_dst + eb, (ee - eb) * 4, cudaMemcpyHostToDevice, c->s_cap2);
+                e = cudaMemcpyAsync(cv.slot_dst[L], c->h_dst + sd.w0, sd.n * 4, cudaMemcpyHostToDevice, c->s_cap2);
                 if (e == cudaSuccess && n_arrays == 2)
-                    e = cudaMemcpyAsync(cv.slot_w[L], c->h_w + eb, (ee - eb) * 4, cudaMemcpyHostToDevice, c->s_cap2);
+                    e = cudaMemcpyAsync(cv.slot_w[L], c->h_w + sw.w0, sw.n * 4, cudaMemcpyHostToDevice, c->s_cap2);
             } else {
-                e = launch_copy_words(c->m_dst + e0, cv.slot_dst[L], ee - e0, c->d_loop, c->s_cap2);
+                e = launch_copy_words(c->m_dst + sd.w0, cv.slot_dst[L], sd.n, c->d_loop, c->s_cap2);
                 if (e == cudaSuccess && n_arrays == 2)
-                    e = launch_copy_words(c->m_w + e0, cv.slot_w[L], ee - e0, c->d_loop, c->s_cap2);
+                    e = launch_copy_words(c->m_w + sw.w0, cv.slot_w[L], sw.n, c->d_loop, c->s_cap2);
                 c->loop_kernels += n_arrays;
             }
             RelaxTask t{};
-            t.route = kRouteF; t.mode = kModeDevice; t.dst = cv.slot_dst[L]; t.w = cv.slot_w[L];
-            t.shift = (long long)e0; t.src_len = ee - e0;
+            t.route = kRouteF; t.mode = kModeDevice; t.src = slot_edges(c, L, eb, ee - eb);
             t.dev_edge = pa.route_edge + i; t.dev_len = pa.edges + i; t.dev_entry = pa.route_entry + i;
             const bool again = second_pass_on(c, algo) &&
                                range_second_pass(c, ee - eb, c->part_vb[i + 1] - c->part_vb[i]);
@@ -1311,8 +1409,7 @@ hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::ve
             }
             if (e == cudaSuccess && again) {
                 ScopedTime tm(c, kKindSecondPass, c->s_cap2);
-                e = second_pass_any(c, st, cv.slot_dst[L], cv.slot_w[L], (long long)e0, ee - e0, i, i + 1, c->d_sp,
-                                    c->s_cap2);
+                e = second_pass_any(c, st, t.src, i, i + 1, c->d_sp, c->s_cap2);
                 count_second_launch(c);
             }
         }
@@ -1334,13 +1431,13 @@ hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::ve
         c->loop_ch = (unsigned long long)h;
         CK(cudaStreamBeginCaptureToGraph(c->s_cap2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         RelaxTask gt{};
-        gt.route = kRouteC; gt.mode = kModeHost; gt.dst = c->m_dst; gt.w = c->m_w; gt.shift = 0;
-        gt.device_sized = true; gt.src_len = c->E; gt.link_ctr = c->d_link_ctr + 2 * kRouteC;
+        gt.route = kRouteC; gt.mode = kModeHost; gt.src = host_edges(c);
+        gt.device_sized = true; gt.link_ctr = c->d_link_ctr + 2 * kRouteC;
         cudaError_t e = launch_gather(la, sum, gt, cv.cmp_dst, n_arrays == 2 ? cv.cmp_w : nullptr, cap, c->s_cap2,
                                       c->d_loop);
         RelaxTask rt{};
-        rt.route = kRouteC; rt.mode = kModeCompact; rt.dst = cv.cmp_dst; rt.w = cv.cmp_w; rt.shift = 0;
-        rt.device_sized = true; rt.src_len = cv.compact_edges;
+        rt.route = kRouteC; rt.mode = kModeCompact; rt.src = compact_edges(c, 0, cv.compact_edges);
+        rt.device_sized = true;
         if (e == cudaSuccess) e = relax_any(c, st, la, sum, rt, cap, c->s_cap2);
         cudaGraph_t captured = nullptr;
         const cudaError_t e_end = cudaStreamEndCapture(c->s_cap2, &captured);
@@ -1491,10 +1588,12 @@ hytg_status ensure_cache(hytg_ctx *c, int n_arrays) {
     if (c->cache_filled_arrays == n_arrays && c->cache_filled_n == cv.n_cached) return HYTG_OK;
     if (cv.cache_edges) {
         ScopedTime t(c, HYTG_K_CACHE_FILL, c->s_main);
-        CK(cudaMemcpyAsync(cv.cache_dst, c->h_dst, cv.cache_edges * 4, cudaMemcpyHostToDevice, c->s_main));
+        CK(cudaMemcpyAsync(cv.cache_dst, c->h_dst, word_span(0, cv.cache_edges, c->dst_bits).n * 4,
+                           cudaMemcpyHostToDevice, c->s_main));
         if (n_arrays == 2)
-            CK(cudaMemcpyAsync(cv.cache_w, c->h_w, cv.cache_edges * 4, cudaMemcpyHostToDevice, c->s_main));
-        c->stats.cache_fill_bytes += cv.cache_edges * 4 * n_arrays;
+            CK(cudaMemcpyAsync(cv.cache_w, c->h_w, word_span(0, cv.cache_edges, c->w_bits).n * 4,
+                               cudaMemcpyHostToDevice, c->s_main));
+        c->stats.cache_fill_bytes += copy_bytes(c, 0, cv.cache_edges, n_arrays);
     }
     c->cache_filled_arrays = n_arrays;
     c->cache_filled_n = cv.n_cached;
@@ -1572,8 +1671,9 @@ hytg_status host_compact(hytg_ctx *c, int algo, unsigned int bucket, const Summa
                 const uint64_t take = std::min<uint64_t>(e_hi, z) - pos;
                 const uint64_t src = h_soff[i] + (pos - h_ebase[i]);
                 if (e_hi <= pos || src + take > E) { bad = 1; return; }
-                std::memcpy(sd + (pos - cb), hd + src, take * 4);
-                if (n_arrays == 2) std::memcpy(sw + (pos - cb), hw + src, take * 4);
+                for (uint64_t j = 0; j < take; ++j) sd[pos - cb + j] = packed_get(hd, c->dst_bits, src + j);
+                if (n_arrays == 2)
+                    for (uint64_t j = 0; j < take; ++j) sw[pos - cb + j] = packed_get(hw, c->w_bits, src + j);
                 pos += take;
             }
         };
@@ -1588,10 +1688,9 @@ hytg_status host_compact(hytg_ctx *c, int algo, unsigned int bucket, const Summa
         }
         CK(cudaEventRecord(c->ev_cstage[b], c->s_c));
         RelaxTask r{};
-        r.route = kRouteC; r.mode = kModeCompact; r.dst = cv.cmp_dst; r.w = cv.cmp_w;
-        r.shift = (long long)cb; r.k_begin = cb; r.k_end = ce; r.first_entry = 0;
+        r.route = kRouteC; r.mode = kModeCompact; r.src = compact_edges(c, cb, ce);
+        r.k_begin = cb; r.k_end = ce; r.first_entry = 0;
         r.device_sized = false;
-        r.src_len = ce - cb;
         {
             ScopedTime tm(c, HYTG_K_RELAX_C, c->s_c);
             CK(relax_any(c, st, la, dsum, r, 8 * (int)device_sms(), c->s_c));
@@ -1713,29 +1812,20 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
     const uint32_t n_fs = std::max<uint32_t>(1, std::min<uint32_t>(cv.n_slots, (uint32_t)c->streams));
     uint32_t rr = ahead ? c->ring_pos : 0;
     int last_copied = -1;                     // slot of this iteration's last copy
-    // An F copy by the copy engine moves the task's edges exactly; the copy
-    // kernel ("f_copy" > 0) starts at the 16-byte boundary at or below the
-    // first edge, so the slot then holds up to 3 words before it (when it has
-    // room for them).  base_of gives the first edge a slot holds for a task.
-    auto by_kernel = [&](uint64_t e0, uint64_t edges) {
-        return c->f_copy > 0 && edges + (e0 & 3) <= cv.slot_edges;
-    };
-    auto base_of = [&](uint64_t e0, uint64_t edges) -> uint64_t {
-        return by_kernel(e0, edges) ? (e0 & ~uint64_t(3)) : e0;
-    };
+    // A copy moves the words that hold the task's edges, from the 16-byte
+    // boundary at or below the first one: by the copy engine, or by a kernel
+    // ("f_copy" > 0).
     auto copy_task = [&](uint32_t slot, uint64_t e0, uint64_t edges, cudaStream_t cs) -> cudaError_t {
-        cudaError_t e;
-        if (by_kernel(e0, edges)) {
-            const uint64_t ea = e0 & ~uint64_t(3);
-            e = launch_stage_copy(c->m_dst + ea, cv.slot_dst[slot], e0 + edges - ea, (unsigned)c->f_copy, cs);
-            if (e == cudaSuccess && n_arrays == 2)
-                e = launch_stage_copy(c->m_w + ea, cv.slot_w[slot], e0 + edges - ea, (unsigned)c->f_copy, cs);
-            c->stats.kernel_launches += n_arrays;
-        } else {
-            e = cudaMemcpyAsync(cv.slot_dst[slot], c->h_dst + e0, edges * 4, cudaMemcpyHostToDevice, cs);
-            if (e == cudaSuccess && n_arrays == 2)
-                e = cudaMemcpyAsync(cv.slot_w[slot], c->h_w + e0, edges * 4, cudaMemcpyHostToDevice, cs);
+        cudaError_t e = cudaSuccess;
+        for (int a = 0; a < n_arrays && e == cudaSuccess; ++a) {
+            const WordSpan sp = word_span(e0, edges, a ? c->w_bits : c->dst_bits);
+            uint32_t *to = a ? cv.slot_w[slot] : cv.slot_dst[slot];
+            if (c->f_copy > 0)
+                e = launch_stage_copy((a ? c->m_w : c->m_dst) + sp.w0, to, sp.n, (unsigned)c->f_copy, cs);
+            else
+                e = cudaMemcpyAsync(to, (a ? c->h_w : c->h_dst) + sp.w0, sp.n * 4, cudaMemcpyHostToDevice, cs);
         }
+        if (c->f_copy > 0) c->stats.kernel_launches += n_arrays;
         return e;
     };
     for (uint32_t k : order) {
@@ -1762,7 +1852,7 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             CK(cudaStreamWaitEvent(cs, c->ev_free[slot], 0));
             {
                 ScopedTime t(c, HYTG_K_COPY_F, cs);
-                t.bytes = (e0 + edges - base_of(e0, edges)) * ebytes;
+                t.bytes = copy_bytes(c, e0, edges, n_arrays);
                 t.part_first = i0;
                 t.part_last = j;
                 CK(copy_task(slot, e0, edges, cs));
@@ -1777,7 +1867,7 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             // the slot's last copy finished before the previous iteration
             // ended (its relax waited for it, and the main stream for that)
             c->stats.f_reused_tasks += 1;
-            c->stats.f_reused_bytes += edges * ebytes;
+            c->stats.f_reused_bytes += copy_bytes(c, e0, edges, n_arrays);
         }
         if (std::find(f_streams_used.begin(), f_streams_used.end(), (int)fi) == f_streams_used.end()) {
             f_streams_used.push_back((int)fi);
@@ -1785,15 +1875,12 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
         }
         // a copy ahead may still be in flight; a reused slot's copy is not
         if (!reuse || ahead) CK(cudaStreamWaitEvent(fs, c->ev_copied[slot], 0));
-        const uint64_t ea = base_of(e0, edges);
         RelaxTask t{};
-        t.route = kRouteF; t.mode = kModeDevice; t.dst = cv.slot_dst[slot]; t.w = cv.slot_w[slot];
-        t.shift = (long long)ea;
+        t.route = kRouteF; t.mode = kModeDevice; t.src = slot_edges(c, slot, e0, edges);
         t.k_begin = p_redge[i0];
         t.k_end = p_redge[j] + p_edges[j];
         t.first_entry = p_rentry[i0];
         t.device_sized = false;
-        t.src_len = e0 + edges - ea;
         const bool again = second_pass_on(c, algo) && range_second_pass(c, edges, c->part_vb[j + 1] - c->part_vb[i0]);
         if (again) t.sp_reset = sp_first_cursor(c, i0);
         {
@@ -1809,13 +1896,12 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             tm.vertices = c->part_vb[j + 1] - c->part_vb[i0];
             tm.part_first = i0;
             tm.part_last = j;
-            CK(second_pass_any(c, st, cv.slot_dst[slot], cv.slot_w[slot], (long long)ea, e0 + edges - ea, i0, j + 1,
-                               ctr, fs));
+            CK(second_pass_any(c, st, t.src, i0, j + 1, ctr, fs));
             count_second_launch(c);
             c->stats.second_pass_vertices += c->part_vb[j + 1] - c->part_vb[i0];
         }
         CK(cudaEventRecord(c->ev_free[slot], fs));
-        if (!reuse) f_bytes += (e0 + edges - ea) * ebytes;
+        if (!reuse) f_bytes += copy_bytes(c, e0, edges, n_arrays);
         ++n_tasks;
     }
     // --- C: gather active lists into the compaction buffer, relax, in chunks
@@ -1828,18 +1914,17 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
         for (uint64_t cb = 0; cb < c_edges; cb += cv.compact_edges) {
             const uint64_t ce = std::min<uint64_t>(c_edges, cb + cv.compact_edges);
             RelaxTask g{};
-            g.route = kRouteC; g.mode = kModeHost; g.dst = c->m_dst; g.w = c->m_w; g.shift = 0;
+            g.route = kRouteC; g.mode = kModeHost; g.src = host_edges(c);
             g.k_begin = cb; g.k_end = ce; g.first_entry = 0; g.device_sized = false;
-            g.src_len = c->E; g.link_ctr = c->d_link_ctr + 2 * kRouteC;
+            g.link_ctr = c->d_link_ctr + 2 * kRouteC;
             {
                 ScopedTime tm(c, HYTG_K_GATHER_C, c->s_c);
                 CK(launch_gather(la, dsum, g, cv.cmp_dst, n_arrays == 2 ? cv.cmp_w : nullptr, 8 * (int)device_sms(), c->s_c));
             }
             RelaxTask r{};
-            r.route = kRouteC; r.mode = kModeCompact; r.dst = cv.cmp_dst; r.w = cv.cmp_w;
-            r.shift = (long long)cb; r.k_begin = cb; r.k_end = ce; r.first_entry = 0;
+            r.route = kRouteC; r.mode = kModeCompact; r.src = compact_edges(c, cb, ce);
+            r.k_begin = cb; r.k_end = ce; r.first_entry = 0;
             r.device_sized = false;
-            r.src_len = ce - cb;
             {
                 ScopedTime tm(c, HYTG_K_RELAX_C, c->s_c);
                 CK(relax_any(c, st, la, dsum, r, 8 * (int)device_sms(), c->s_c));
@@ -1873,10 +1958,10 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             c->slot_held[slot] = hytg_ctx::SlotHeld();
             CK(cudaStreamWaitEvent(cs, c->ev_free[slot], 0));
             if (after) CK(cudaStreamWaitEvent(cs, after, 0));
-            const uint64_t words = e0 + ft.edges - base_of(e0, ft.edges);
+            const uint64_t nbytes = copy_bytes(c, e0, ft.edges, n_arrays);
             {
                 ScopedTime t(c, HYTG_K_COPY_F, cs);
-                t.bytes = words * ebytes;
+                t.bytes = nbytes;
                 t.part_first = ft.i;
                 t.part_last = ft.j;
                 CK(copy_task(slot, e0, ft.edges, cs));
@@ -1885,7 +1970,7 @@ hytg_status issue_work(hytg_ctx *c, int algo, unsigned int bucket, const char *h
             c->slot_held[slot] = {ft.i, ft.j, n_arrays};
             c->ahead.push_back({slot, ft.i, ft.j, n_arrays});
             c->stats.f_ahead_tasks += 1;
-            f_bytes += words * ebytes;
+            f_bytes += nbytes;
         }
         c->ahead_seq = c->work_seq + 1;
     }
@@ -2163,10 +2248,21 @@ hytg_status hytg_load_csr(hytg_ctx *c, uint64_t V, uint64_t E, const uint64_t *o
         free_graph(c);
         if (getenv("HYTG_INJECT_HOSTMEM_FAIL") && atoi(getenv("HYTG_INJECT_HOSTMEM_FAIL")) != 0)
             return fail(c, HYTG_ERR_HOSTMEM, "pinned allocation failure injected by HYTG_INJECT_HOSTMEM_FAIL");
-        const size_t eb = std::max<uint64_t>(E, 1) * 4;
-        if (alloc_edge_array(c, 0, &c->h_dst, eb) != HYTG_OK)
+        // widths of the packed arrays (see EdgeSrc)
+        c->dst_bits = bits_for(V - 1);
+        c->w_bits = 32;
+        if (weights) {
+            std::atomic<uint32_t> any{0};          // OR of the weights: its top bit is the largest one's
+            parallel_chunks(E, [&](uint64_t lo, uint64_t hi) {
+                uint32_t x = 0;
+                for (uint64_t e = lo; e < hi; ++e) x |= weights[e];
+                any |= x;
+            });
+            c->w_bits = bits_for(any);
+        }
+        if (alloc_edge_array(c, 0, &c->h_dst, 4 * packed_words(E, c->dst_bits)) != HYTG_OK)
             return fail(c, HYTG_ERR_HOSTMEM, "pinned allocation of the neighbour array failed");
-        if (weights && alloc_edge_array(c, 1, &c->h_w, eb) != HYTG_OK) {
+        if (weights && alloc_edge_array(c, 1, &c->h_w, 4 * packed_words(E, c->w_bits)) != HYTG_OK) {
             free_graph(c);
             return fail(c, HYTG_ERR_HOSTMEM, "pinned allocation of the weight array failed");
         }
@@ -2183,23 +2279,32 @@ hytg_status hytg_load_csr(hytg_ctx *c, uint64_t V, uint64_t E, const uint64_t *o
                 const uint64_t o = c->h_perm[n];
                 c->h_off[n + 1] = c->h_off[n] + (offsets[o + 1] - offsets[o]);
             }
-            const uint32_t *inv = c->h_inv.data();
-            parallel_chunks(V, [&](uint64_t lo, uint64_t hi) {
-                for (uint64_t n = lo; n < hi; ++n) {
-                    const uint64_t o = c->h_perm[n], s0 = offsets[o], len = offsets[o + 1] - s0;
-                    uint32_t *d = c->h_dst + c->h_off[n];
-                    for (uint64_t j = 0; j < len; ++j) d[j] = inv[dst[s0 + j]];
-                    if (weights) memcpy(c->h_w + c->h_off[n], weights + s0, len * 4);
-                }
-            });
             c->permuted = true;
             c->n_hubs = nh;
         } else {
-            parallel_chunks(E, [&](uint64_t lo, uint64_t hi) {
-                memcpy(c->h_dst + lo, dst + lo, (hi - lo) * 4);
-                if (weights) memcpy(c->h_w + lo, weights + lo, (hi - lo) * 4);
-            });
             c->h_off.assign(offsets, offsets + V + 1);
+        }
+        {
+            // pack the rows in internal order, in pieces of whole groups of 32
+            // edges (a group ends on a word boundary whatever the width)
+            const uint32_t *inv = c->permuted ? c->h_inv.data() : nullptr;
+            const std::vector<uint64_t> &ho = c->h_off;
+            parallel_chunks((E + 31) / 32, [&](uint64_t glo, uint64_t ghi) {
+                const uint64_t lo = glo * 32, hi = std::min<uint64_t>(E, ghi * 32);
+                if (lo >= hi) return;
+                PackedWriter pd(c->h_dst, c->dst_bits, lo), pw(weights ? c->h_w : c->h_dst, c->w_bits, lo);
+                uint64_t n = (uint64_t)(std::upper_bound(ho.begin(), ho.end(), lo) - ho.begin()) - 1;
+                for (uint64_t e = lo; e < hi; ++n) {
+                    const uint64_t end = std::min<uint64_t>(hi, ho[n + 1]);
+                    const uint64_t from = offsets[inv ? c->h_perm[n] : n] + (e - ho[n]), cnt = end > e ? end - e : 0;
+                    for (uint64_t j = 0; j < cnt; ++j) pd.put(inv ? inv[dst[from + j]] : dst[from + j]);
+                    if (weights)
+                        for (uint64_t j = 0; j < cnt; ++j) pw.put(weights[from + j]);
+                    e += cnt;
+                }
+                pd.finish();
+                if (weights) pw.finish();
+            }, 1u << 14);
         }
         void *mp = nullptr;
         CK(cudaHostGetDevicePointer(&mp, c->h_dst, 0));
@@ -2398,7 +2503,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         if (algo == kCC) {
             // checked once per loaded graph, on the internal arrays (hub
             // sorting relabels vertices, which keeps symmetry)
-            if (c->symmetric < 0) c->symmetric = csr_symmetric(c->h_off, c->h_dst, c->V) ? 1 : 0;
+            if (c->symmetric < 0) c->symmetric = csr_symmetric(c->h_off, c->h_dst, c->dst_bits, c->V) ? 1 : 0;
             if (!c->symmetric)
                 return fail(c, HYTG_ERR_ARG,
                             "CC needs a symmetric CSR (every edge u->v with a reverse v->u of the same "
@@ -2906,7 +3011,8 @@ hytg_status hytg_get_info(hytg_ctx *c, hytg_info *out) {
     i.budget_used_bytes = c->carve.used;
     i.compact_edges = c->carve.compact_edges;
     i.vertex_state_bytes = c->loaded ? c->vertex_bytes : 0;
-    i.pinned_host_bytes = c->loaded ? std::max<uint64_t>(c->E, 1) * 4 * (c->weighted ? 2 : 1) : 0;
+    i.pinned_host_bytes = c->loaded ? 4 * (packed_words(c->E, c->dst_bits) +
+                                           (c->weighted ? packed_words(c->E, c->w_bits) : 0)) : 0;
     *out = i;
     return HYTG_OK;
 }

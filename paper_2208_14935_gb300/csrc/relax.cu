@@ -7,11 +7,10 @@
 // adjacent lists: 128-byte lines when the lists are long, and neighbouring
 // lists share lines when consecutive vertices are active.
 //
-// Edge sources (the route's transfer method):
+// Edge sources (the route's transfer method; packed as EdgeSrc says):
 //   host    zero-copy loads from pinned, device-mapped host memory (Eq. 3 route);
-//   device  a device copy starting at CSR edge `shift` (cache and F routes:
-//           the partition's edges are shifted by its first edge index);
-//   compact the compacted buffer, where route edge k sits at k - shift.
+//   device  a device copy of a run of edges (cache and F routes);
+//   compact the compaction buffer: plain words in route order.
 #include "common.cuh"
 #include "edge_runs.cuh"
 
@@ -64,15 +63,9 @@ template <int ALGO>
 __device__ __forceinline__ void relax_edges(const AlgoState &st, const RelaxTask &t,
                                             const Edge<false> (&ed)[kSteps], float *hub_rep) {
     constexpr bool rank = ALGO == kPR || ALGO == kPPR;
-    unsigned int dv[kSteps], wv[kSteps], cur[kSteps];
-#pragma unroll
-    for (int q = 0; q < kSteps; ++q) {
-        dv[q] = wv[q] = 0;
-        if (ed[q].ok) {
-            dv[q] = __ldg(t.dst + ed[q].e);
-            if (ALGO == kSSSP) wv[q] = __ldg(t.w + ed[q].e);
-        }
-    }
+    unsigned int dv[kSteps], wv[kSteps] = {}, cur[kSteps];
+    load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
+    if (ALGO == kSSSP) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
     if (!rank) {
         // the values are read together before any reduction is issued (a
         // reduction between them would make the loads wait for one another)
@@ -92,10 +85,11 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax(AlgoState st, ListArrays 
     const RouteView rv = task_view(t, sum, kb, ke);
     float *hub_rep = st.hub_rep ? st.hub_rep + (size_t)(sm_id() % kHubReplicas) * st.n_hub_rep : nullptr;
     LinkCount lc;
+    lc.weights = ALGO == kSSSP;
     walk_task<kSteps, false>(la, rv, t, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long) {
         relax_edges<ALGO>(st, t, ed, hub_rep);
     });
-    flush_link(lc, ALGO == kSSSP ? 2u : 1u, t.link_ctr);
+    flush_link(lc, t.link_ctr);
 }
 
 // Two device-sized routes in one launch (cache and zero-copy in the device
@@ -114,6 +108,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_pair(AlgoState st, ListAr
     const int sh = run_shift(ea + eb, nwarps);
     const unsigned long long na = (ea + (1ull << sh) - 1) >> sh, nb = (eb + (1ull << sh) - 1) >> sh;
     LinkCount la_ct, lb_ct;
+    la_ct.weights = lb_ct.weights = ALGO == kSSSP;
     const auto body = [&](const RelaxTask &t) {
         return [&st, &t, hub_rep](const Edge<false> (&ed)[kSteps], unsigned long long) {
             relax_edges<ALGO>(st, t, ed, hub_rep);
@@ -123,8 +118,8 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_pair(AlgoState st, ListAr
         if (r < na) walk_run<kSteps, false>(la, va, ta, r, sh, 0ull, ea, la_ct, body(ta));
         else walk_run<kSteps, false>(la, vb, tb, r - na, sh, 0ull, eb, lb_ct, body(tb));
     }
-    flush_link(la_ct, ALGO == kSSSP ? 2u : 1u, ta.link_ctr);
-    flush_link(lb_ct, ALGO == kSSSP ? 2u : 1u, tb.link_ctr);
+    flush_link(la_ct, ta.link_ctr);
+    flush_link(lb_ct, tb.link_ctr);
 }
 
 __global__ void __launch_bounds__(kRelaxBlock) k_gather(ListArrays la, const Summary *sum,
@@ -134,16 +129,11 @@ __global__ void __launch_bounds__(kRelaxBlock) k_gather(ListArrays la, const Sum
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     LinkCount lc;
+    lc.weights = out_w != nullptr;
     walk_task<kSteps, false>(la, rv, t, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long k) {
-        unsigned int dv[kSteps], wv[kSteps];
-#pragma unroll
-        for (int q = 0; q < kSteps; ++q) {
-            dv[q] = wv[q] = 0;
-            if (ed[q].ok) {
-                dv[q] = __ldg(t.dst + ed[q].e);
-                if (out_w) wv[q] = __ldg(t.w + ed[q].e);
-            }
-        }
+        unsigned int dv[kSteps], wv[kSteps] = {};
+        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
+        if (out_w) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
 #pragma unroll
         for (int q = 0; q < kSteps; ++q) {
             if (ed[q].ok) {
@@ -152,7 +142,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_gather(ListArrays la, const Sum
             }
         }
     });
-    flush_link(lc, out_w ? 2u : 1u, t.link_ctr);
+    flush_link(lc, t.link_ctr);
 }
 
 // Second pass over a resident vertex range (Sec. VI-A: a loaded subgraph is
