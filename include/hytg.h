@@ -233,7 +233,11 @@ hytg_status hytg_set_device_budget(hytg_ctx *ctx, uint64_t bytes);
  * partition order, which hub sorting makes hub-first), "device_loop" (1,
  * default: runs replay one iteration (planning, binning, cache and zero-copy
  * relax) inside a CUDA graph with a WHILE node; a single-source iteration
- * that needs the F or C route goes to the host, which issues its copies,
+ * that needs the F or C route goes to the host, which issues its copies
+ * (BFS, SSSP and CC iterations with up to 4,096 active vertices and 16,384
+ * edges, no F route and at most 1,024 partitions run several at a time in one
+ * kernel of the body, the C route's lists read from mapped host memory there
+ * unless "compact_host" is on),
  * while batched runs keep F and C iterations in the graph too: one IF node
  * per partition copies it into a staging slot and relaxes it, one IF node
  * gathers and relaxes the C route, each F copy moves one partition (no task

@@ -164,7 +164,21 @@ struct LoopCtl {
     unsigned long long route_parts[kRoutes], route_entries[kRoutes], route_edges[kRoutes];
     unsigned long long z_lines, vertices, edges, iterations;
     unsigned long long f_parts, f_bytes, c_iters, c_lines;
+    // small-frontier iterations (k_tail): allowed in this graph, chosen for the
+    // iteration being planned, the first iteration it may take after one that
+    // it refused, iterations it has run; body runs (each launches the whole body)
+    unsigned int tail_ok, tail_gather, tail, tail_not;
+    unsigned long long tail_its, bodies;
 };
+
+// Small-frontier iterations: queue entries (a thread each), partitions whose
+// routes one block decides, and the frontier that k_select hands over.  A
+// 1021 x 1031 mesh (CC, device time): frontiers up to 2,048 vertices 26.2 ms,
+// up to the whole queue 19.3 ms; more edges than 4 a thread gain nothing on
+// meshes and make R-MAT frontiers (a few lists of thousands of edges) try in
+// vain.
+constexpr unsigned int kTailQueue = 4096, kTailParts = 1024, kTailActive = 4096, kTailEdges = 16384;
+enum TailExit : int { kTailAgain = 0, kTailDone = 1, kTailMaxIt = 2, kTailCancel = 3 };
 
 struct AlgoState {
     int algo;
@@ -246,6 +260,13 @@ __device__ __forceinline__ void ppr_push_vec(const BatchState &b, unsigned long 
 }
 constexpr unsigned int kHubReplicas = 256;
 
+// log2 of a power of two, else -1.
+inline int log2_exact(unsigned long long m) {
+    if (m == 0 || (m & (m - 1))) return -1;
+    int s = 0;
+    while ((1ull << s) < m) ++s;
+    return s;
+}
 cudaError_t launch_count(const GraphDev &g, const AlgoState &st, const PartArrays &pa,
                          unsigned long long m, cudaStream_t s);
 // With ctl, the device loop's decision too: cond is the WHILE node's condition.
@@ -300,6 +321,22 @@ struct RelaxTask {
 
 // Cursor of a second pass's list: entries in the low 30 bits, edges above.
 constexpr unsigned long long kSpEntries = (1ull << 30) - 1, kSpEdgesMax = (1ull << 34) - 1;
+
+struct TailArgs {
+    GraphDev g;
+    AlgoState st;
+    EdgeSrc cache, host;
+    CostParams cp;
+    unsigned long long m;               // request bytes
+    int m_shift;                        // log2 of m when it is a power of two, else -1
+    int gather;                         // 1: the compaction route runs here too
+    LoopCtl *ctl;
+    unsigned int *queue[2];             // kTailQueue vertices each
+    unsigned long long *link_ctr;       // per route {sectors, lines}
+    unsigned int *err;
+    unsigned long long cond;            // the WHILE node's condition
+};
+cudaError_t launch_tail(const TailArgs &a, cudaStream_t s);
 
 cudaError_t launch_relax(const AlgoState &st, const ListArrays &la, const Summary *sum,
                          const RelaxTask &t, int grid_cap, cudaStream_t s);

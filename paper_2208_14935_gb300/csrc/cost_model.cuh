@@ -7,7 +7,13 @@
 
 namespace hytg {
 
+// ceil(x / d); by shifts when d is a power of two, as the paper's m and MR are
+// (the decision is on the critical path of every iteration).
 __device__ __forceinline__ unsigned long long div_up(unsigned long long x, unsigned long long d) {
+    if ((d & (d - 1)) == 0) {
+        const int s = __ffsll((long long)d) - 1;
+        return (x >> s) + ((x & (d - 1)) != 0);
+    }
     const unsigned long long q = x / d;
     return q + (x != q * d);
 }

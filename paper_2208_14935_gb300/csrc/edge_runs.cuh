@@ -124,20 +124,20 @@ template <int S, class E>
 __device__ __forceinline__ void load_entries(const unsigned int *p, unsigned int bits, long long off,
                                              const E (&ed)[S], unsigned int (&out)[S]) {
     const unsigned int mask = 0xffffffffu >> (32 - bits);
-    unsigned int lo[S], sh[S];
-    long long at[S];
+    unsigned int lo[S], hi[S], sh[S];
 #pragma unroll
     for (int q = 0; q < S; ++q) {
         const long long bit = ed[q].ok ? ed[q].e * (long long)bits - off : 0;
-        at[q] = bit >> 5;
+        const unsigned int *at = p + (bit >> 5);
         sh[q] = (unsigned int)bit & 31u;
-        lo[q] = ed[q].ok ? __ldg(p + at[q]) : 0u;
+        lo[q] = ed[q].ok ? __ldg(at) : 0u;
+        // beside the first word's load, not behind it
+        hi[q] = ed[q].ok && !ed[q].adj && sh[q] + bits > 32 ? __ldg(at + 1) : 0u;
     }
 #pragma unroll
     for (int q = 0; q < S; ++q) {
-        unsigned int hi = __shfl_down_sync(0xffffffffu, lo[q], 1);
-        if (ed[q].ok && !ed[q].adj && sh[q] + bits > 32) hi = __ldg(p + at[q] + 1);
-        out[q] = ed[q].ok ? __funnelshift_r(lo[q], hi, sh[q]) & mask : 0u;
+        const unsigned int next = __shfl_down_sync(0xffffffffu, lo[q], 1);
+        out[q] = ed[q].ok ? __funnelshift_r(lo[q], ed[q].adj ? next : hi[q], sh[q]) & mask : 0u;
     }
 }
 

@@ -312,12 +312,14 @@ struct hytg_ctx {
     uint32_t loop_f_kernels = 0, loop_c_kernels = 0;
     bool loop_fc = false;                                // the captured body holds F and C nodes
     int last_run_arrays = 1;                             // edge arrays the current run reads
+    int last_run_algo = 0;                               // algorithm of the current run
     int loop_fc_copy = 0;                                // 0 memcpy nodes, 1 copy kernel, 2 not available
 
     cudaGraph_t loop_graph = nullptr;
     cudaGraphExec_t loop_exec = nullptr;
     std::string loop_key;                                // what the captured body depends on
     LoopCtl *d_loop = nullptr, *h_loop = nullptr;        // device control block, pinned mirror
+    unsigned int *d_tail_q = nullptr;                    // two queues of small-frontier iterations
     unsigned int *h_cancel = nullptr, *d_cancel = nullptr;  // mapped word: end the device loop
     bool has_deadline = false;
     std::chrono::steady_clock::time_point run_deadline;
@@ -1449,6 +1451,34 @@ hytg_status capture_loop_fc(hytg_ctx *c, int algo, cudaGraph_t cg, const std::ve
     return HYTG_OK;
 }
 
+// Small-frontier iterations (k_tail) apply to single-source BFS, SSSP and CC
+// with few enough partitions for one block to route.
+bool tail_applies(const hytg_ctx *c, int algo) {
+    return c->batch_mode == kBatchNone && (algo == kBFS || algo == kSSSP || algo == kCC) &&
+           !second_pass_on(c, algo) && c->part_vb.size() - 1 <= kTailParts;
+}
+
+hytg_status capture_tail(hytg_ctx *c, int algo, cudaStream_t s, unsigned long long handle) {
+    TailArgs a{};
+    a.g = graph_dev(c);
+    a.st = algo_state(c, algo);
+    a.cache = cache_edges(c);
+    a.host = host_edges(c);
+    a.cp = cost_params(c, algo, 1);
+    a.m = (unsigned long long)c->m;
+    a.ctl = c->d_loop;
+    a.queue[0] = c->d_tail_q;
+    a.queue[1] = c->d_tail_q + kTailQueue;
+    a.m_shift = log2_exact(a.m);
+    a.gather = c->compact_host == 0;
+    a.link_ctr = c->d_link_ctr;
+    a.err = c->d_err;
+    a.cond = handle;
+    ScopedTime t(c, HYTG_K_OTHER, s);
+    CK(launch_tail(a, s));
+    return HYTG_OK;
+}
+
 hytg_status capture_loop_body(hytg_ctx *c, int algo, cudaStream_t s, unsigned long long handle) {
     GraphDev g = graph_dev(c);
     AlgoState st = algo_state(c, algo);
@@ -1495,9 +1525,9 @@ hytg_status ensure_loop_graph(hytg_ctx *c, int algo) {
                   (void *)c->bs.val[0]);
     {
         const size_t n = std::strlen(key);
-        std::snprintf(key + n, sizeof key - n, "|fc%d.%d|%u|%p|%p|%llu", (int)c->loop_fc, c->loop_fc_copy,
+        std::snprintf(key + n, sizeof key - n, "|fc%d.%d|%u|%p|%p|%llu|%d", (int)c->loop_fc, c->loop_fc_copy,
                       c->carve.n_slots, (void *)c->carve.slot_dst[0], (void *)c->carve.cmp_dst,
-                      (unsigned long long)c->carve.compact_edges);
+                      (unsigned long long)c->carve.compact_edges, c->compact_host == 0);
     }
     if (c->loop_exec && c->loop_key == key) return HYTG_OK;
     free_loop_graph(c);
@@ -1526,6 +1556,8 @@ hytg_status ensure_loop_graph(hytg_ctx *c, int algo) {
         c->capturing = true;
         hytg_status st = piece == 0 ? capture_loop_body(c, algo, c->s_cap, (unsigned long long)h)
                                     : issue_plan_tail(c, algo, 0xFFFFFFFFu, c->s_cap, c->d_loop, 2);
+        if (st == HYTG_OK && piece == 1 && tail_applies(c, algo))
+            st = capture_tail(c, algo, c->s_cap, (unsigned long long)h);
         if (st == HYTG_OK && piece == 0) {
             cudaStreamCaptureStatus cs;
             const cudaGraphNode_t *deps = nullptr;
@@ -2043,6 +2075,8 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
     h.max_it = (unsigned long long)c->max_iters;
     h.m = (unsigned long long)c->m;
     h.rec = c->d_loop_rec;
+    h.tail_ok = tail_applies(c, c->last_run_algo) ? 1u : 0u;
+    h.tail_gather = c->compact_host == 0 ? 1u : 0u;
     if (c->loop_fc) {
         const PartArrays pa = part_arrays(c);
         h.f_handles = c->d_loop_fh;
@@ -2101,7 +2135,7 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
     c->stats.graph_launches += 1;
     c->stats.graph_iterations += h.iterations;
     // every body run launches the whole body; gated kernels return at once
-    c->stats.kernel_launches += (uint64_t)c->loop_kernels * ((uint64_t)(h.it - it) + 1) +
+    c->stats.kernel_launches += (uint64_t)c->loop_kernels * h.bodies +
                                 h.f_parts * c->loop_f_kernels + h.c_iters * c->loop_c_kernels;
     it = h.it;
     bucket = h.bucket;
@@ -2162,6 +2196,7 @@ hytg_status hytg_create(hytg_ctx **out, int device) {
     ck(cudaStreamCreateWithFlags(&c->s_cap2, cudaStreamNonBlocking));
     ck(cudaMalloc(&c->d_loop_fh, 1024 * sizeof(unsigned long long)));
     ck(cudaMalloc(&c->d_loop, sizeof(LoopCtl)));
+    ck(cudaMalloc(&c->d_tail_q, 2 * kTailQueue * sizeof(unsigned int)));
     ck(cudaMalloc(&c->d_loop_rec, (size_t)c->loop_rec_cap * sizeof(hytg_iter_record)));
     ck(cudaHostAlloc((void **)&c->h_loop, sizeof(LoopCtl), cudaHostAllocDefault));
     ck(cudaHostAlloc((void **)&c->h_cancel, sizeof(unsigned int), cudaHostAllocMapped));
@@ -2205,6 +2240,7 @@ hytg_status hytg_destroy(hytg_ctx *c) {
     for (int i = 0; i < 2; ++i) if (c->ev_run[i]) cudaEventDestroy(c->ev_run[i]);
     free_loop_graph(c);
     dfree(c->d_loop);
+    dfree(c->d_tail_q);
     dfree(c->d_loop_rec);
     if (c->h_loop) cudaFreeHost(c->h_loop);
     if (c->h_cancel) cudaFreeHost(c->h_cancel);
@@ -2533,6 +2569,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         }
         const int n_arrays = (algo == kSSSP) ? 2 : 1;
         c->last_run_arrays = n_arrays;
+        c->last_run_algo = algo;
         CK(cudaEventRecord(c->ev_run[0], c->s_main));
         hytg_status s = plan_carve(c, n_arrays);
         if (s != HYTG_OK) return s;

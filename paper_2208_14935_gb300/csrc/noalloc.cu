@@ -183,9 +183,7 @@ extern "C" hytg_status hytg_plan_noalloc(hytg_algo algo, const uint32_t *frontie
     in.n_parts = n_parts;
     in.n_arrays = a == kSSSP ? 2u : 1u;
     in.m = prm.m;
-    in.m_shift = -1;
-    if ((prm.m & (prm.m - 1)) == 0)
-        for (in.m_shift = 0; (1ull << in.m_shift) < prm.m;) ++in.m_shift;
+    in.m_shift = log2_exact(prm.m);
     // One block per partition while a partition's words are few (up to 64 on
     // average; a warp takes 32 per turn of its block, and skewed graphs have
     // partitions of many times the average) or the partitions alone fill the

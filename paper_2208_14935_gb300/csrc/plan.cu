@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(kSelectBlock) k_select(GraphDev g, PartArrays 
         pa.route_entry[p] = re;
         pa.route_edge[p] = rg;
     }
+    __shared__ Summary s_sum;                       // the summary, also read by the decision
     if (tid < kRoutes) {
         // thread r writes route r's totals and bases
         const unsigned int r = tid;
@@ -285,29 +286,31 @@ __global__ void __launch_bounds__(kSelectBlock) k_select(GraphDev g, PartArrays 
             }
             parts += s_tot[11 + q];
         }
-        sum->route_entries[r] = r ? s_tot[r - 1] : 0ull;
-        sum->route_edges[r] = r ? s_tot[3 + r] : 0ull;
-        sum->route_lines[r] = r ? s_tot[7 + r] : 0ull;
-        sum->route_parts[r] = (unsigned int)(r ? s_tot[11 + r] : N - parts);
-        sum->route_entry_base[r] = e;
-        sum->route_tile_base[r] = t;
+        s_sum.route_entries[r] = r ? s_tot[r - 1] : 0ull;
+        s_sum.route_edges[r] = r ? s_tot[3 + r] : 0ull;
+        s_sum.route_lines[r] = r ? s_tot[7 + r] : 0ull;
+        s_sum.route_parts[r] = (unsigned int)(r ? s_tot[11 + r] : N - parts);
+        s_sum.route_entry_base[r] = e;
+        s_sum.route_tile_base[r] = t;
     }
     if (tid == kRoutes) {
-        sum->n_active = s_tot[16];
-        sum->pending = *pa.pending;
-        sum->pending_min = ~(unsigned int)(*pa.pending_inv);
-        sum->alive = pa.alive ? *pa.alive : 0ull;
+        s_sum.n_active = s_tot[16];
+        s_sum.pending = *pa.pending;
+        s_sum.pending_min = ~(unsigned int)(*pa.pending_inv);
+        s_sum.alive = pa.alive ? *pa.alive : 0ull;
     }
-    if (ctl) {
-        __syncthreads();
-        loop_decide(sum, ctl, cond);
-    }
+    __syncthreads();
+    for (unsigned int i = tid; i < sizeof(Summary) / 4; i += nt)
+        reinterpret_cast<unsigned int *>(sum)[i] = reinterpret_cast<const unsigned int *>(&s_sum)[i];
+    if (ctl) loop_decide(&s_sum, ctl, cond);
 }
 
 // ------------------------------------------------------ device loop
 // Thread 0: the host loop's decisions for the iteration just planned.
 __device__ void loop_decide_one(const Summary *sum, LoopCtl *ctl, cudaGraphConditionalHandle h) {
     ctl->work = 0;
+    ctl->tail = 0;
+    ++ctl->bodies;
     if (sum->n_active == 0) {
         if (sum->pending == 0) {
             ctl->status = kLoopDone;
@@ -334,6 +337,15 @@ __device__ void loop_decide_one(const Summary *sum, LoopCtl *ctl, cudaGraphCondi
         cudaGraphSetConditional(h, 0);
         return;
     }
+    unsigned long long act = 0;
+    for (int q = 0; q < kRoutes; ++q) act += sum->route_edges[q];
+    if (ctl->tail_ok && ctl->it >= ctl->tail_not && ctl->n_rec < ctl->rec_cap && sum->n_active <= kTailActive &&
+        act <= kTailEdges && sum->n_active + sum->pending <= kTailQueue && sum->route_parts[kRouteF] == 0 &&
+        (sum->route_parts[kRouteC] == 0 || ctl->tail_gather)) {
+        ctl->tail = 1;                    // k_tail runs it, and those that follow
+        cudaGraphSetConditional(h, 1);
+        return;
+    }
     const bool f_host = sum->route_parts[kRouteF] != 0 && !ctl->f_handles;
     const bool c_host = sum->route_parts[kRouteC] != 0 &&
                         (!ctl->c_handle || sum->route_edges[kRouteC] > ctl->c_cap);
@@ -343,9 +355,7 @@ __device__ void loop_decide_one(const Summary *sum, LoopCtl *ctl, cudaGraphCondi
         return;
     }
     hytg_iter_record *r = (hytg_iter_record *)ctl->rec + ctl->n_rec++;
-    unsigned long long act = 0;
     for (int q = 0; q < kRoutes; ++q) {
-        act += sum->route_edges[q];
         r->route_partitions[q] = sum->route_parts[q];
         r->route_edges[q] = sum->route_edges[q];
         ctl->route_parts[q] += sum->route_parts[q];
@@ -598,10 +608,7 @@ cudaError_t launch_count(const GraphDev &g, const AlgoState &st, const PartArray
     if (g.n_words_alloc == 0) return cudaSuccess;
     static const unsigned long long resident = resident_blocks(k_count);
     const WalkGrid w = walk_grid(g.n_words_alloc, resident);
-    int m_shift = -1;
-    if ((m & (m - 1)) == 0)
-        for (m_shift = 0; (1ull << m_shift) < m;) ++m_shift;
-    k_count<<<w.blocks, 256, 0, s>>>(g, st, pa, m, m_shift, w.cw);
+    k_count<<<w.blocks, 256, 0, s>>>(g, st, pa, m, log2_exact(m), w.cw);
     return cudaGetLastError();
 }
 
