@@ -304,6 +304,14 @@ hytg_status hytg_run(hytg_ctx *ctx, hytg_algo algo, const uint32_t *sources, uin
  * HYTG_ERR_STATE if no run completed. */
 hytg_status hytg_fetch_result(hytg_ctx *ctx, void *out, uint64_t out_bytes);
 
+/* hytg_run, then hytg_fetch_result into `out` if it succeeded, in one call:
+ * host threads of the context fault in the pages of `out` (their contents
+ * stay) while the run is on the device, so that the copy does not take the
+ * page faults of a fresh allocation one at a time.  `out` must stay valid
+ * until the call returns; arguments and errors are those of the two calls. */
+hytg_status hytg_run_fetch(hytg_ctx *ctx, hytg_algo algo, const uint32_t *sources, uint32_t n_sources,
+                           void *out, uint64_t out_bytes);
+
 /* Raw delta-PageRank state of the last PageRank/PPR run: rank and the
  * residual delta per vertex (float, V entries each; either may be NULL). */
 hytg_status hytg_fetch_pagerank_state(hytg_ctx *ctx, float *rank, float *delta, uint64_t V);

@@ -16,6 +16,7 @@
 // The next iteration's planning kernels wait, on the device, for every
 // stream of the previous one, so the host only blocks on the summary copy.
 #include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <chrono>
@@ -119,6 +120,94 @@ private:
     bool stop_ = false;
 };
 
+// Host threads that fault in the pages of a result buffer while the run that
+// fills it is on the device.  A caller's fresh allocation has no pages yet, and
+// a device-to-host copy into it spends most of its time on page faults taken
+// one at a time (256 MiB: 9.6 ms, against 1.4 ms into present pages; 64 MiB: 2.6
+// and 0.37 ms).  The pages are populated for writing by the kernel call for
+// that, which leaves their contents alone; reading a byte and writing it back
+// would map the zero page first and then replace it, and that replacement,
+// which the device's view of the page tables must follow, made a 64-source BFS
+// take 106 ms instead of 15.  Whole calls, faults in the copy -> after the run
+// from eight threads -> beside the run: 64-source BFS on R-MAT 20 14.8 ->
+// 11.3 -> 8.3 ms, BFS on R-MAT 24 7.9 -> 6.6 -> 5.1 ms.  start() returns at
+// once; finish() helps, and returns when every page is present.
+class PageToucher {
+public:
+    explicit PageToucher(unsigned n) {
+        for (unsigned i = 0; i < n; ++i) th_.emplace_back([this] { loop(); });
+    }
+    ~PageToucher() {
+        { std::lock_guard<std::mutex> l(mu_); stop_ = true; }
+        go_.notify_all();
+        for (auto &t : th_) t.join();
+    }
+    void start(void *p, size_t bytes) {
+        {
+            std::lock_guard<std::mutex> l(mu_);
+            p_ = (char *)p;
+            bytes_ = bytes;
+            next_ = 0;
+            open_ = true;
+            ++gen_;
+        }
+        go_.notify_all();
+    }
+    void finish() {
+        work();
+        std::unique_lock<std::mutex> l(mu_);
+        open_ = false;
+        done_.wait(l, [&] { return active_ == 0; });
+    }
+
+private:
+    static constexpr size_t kPiece = size_t(1) << 21;
+    static constexpr int kPopulateWrite = 23;        // MADV_POPULATE_WRITE (Linux 5.14)
+    void work() {
+        static const size_t page = (size_t)std::max<long>(4096, sysconf(_SC_PAGESIZE));
+        for (;;) {
+            const size_t lo = next_.fetch_add(kPiece);
+            if (lo >= bytes_) return;
+            const size_t hi = std::min(bytes_, lo + kPiece);
+            const uintptr_t a = ((uintptr_t)p_ + lo) & ~(uintptr_t)(page - 1);
+            madvise((void *)a, (uintptr_t)p_ + hi - a, kPopulateWrite);
+        }
+    }
+    void loop() {
+        uint64_t seen = 0;
+        std::unique_lock<std::mutex> l(mu_);
+        for (;;) {
+            go_.wait(l, [&] { return stop_ || (open_ && gen_ != seen); });
+            if (stop_) return;
+            seen = gen_;
+            ++active_;
+            l.unlock();
+            work();
+            l.lock();
+            if (--active_ == 0) done_.notify_one();
+        }
+    }
+    std::vector<std::thread> th_;
+    std::mutex mu_;
+    std::condition_variable go_, done_;
+    char *p_ = nullptr;
+    size_t bytes_ = 0;
+    std::atomic<size_t> next_{0};
+    uint64_t gen_ = 0;
+    unsigned active_ = 0;
+    bool open_ = false, stop_ = false;
+};
+
+// What a run reports besides its result, in one device block, so that one
+// memset clears it and one copy brings it back.
+struct RunReport {
+    unsigned int overflow, err;
+    double prsums[2];
+    unsigned long long src_work;
+    unsigned long long link_ctr[2 * kRoutes];
+    unsigned long long sp[kSpSlots];
+};
+
 struct Carve {
     int n_arrays = 0;           // 0: not planned
     uint64_t budget = 0, part_edges = 0;
@@ -178,7 +267,8 @@ struct hytg_ctx {
     unsigned int *d_vid = nullptr;
     void *d_bout = nullptr;                              // K x V results
     uint32_t bout_rows = 0;                              // rows of V results d_bout holds
-    unsigned long long *d_src_work = nullptr;
+    RunReport *d_report = nullptr, *h_report = nullptr;  // device block, pinned copy
+    unsigned long long *d_src_work = nullptr;            // the following point into d_report
     double *d_bsums = nullptr;
     unsigned long long *d_alive = nullptr;
     unsigned long long *d_sp = nullptr;                  // second-pass edge counters (kSpSlots)
@@ -291,6 +381,8 @@ struct hytg_ctx {
     std::vector<std::pair<size_t, cudaEvent_t>> iter_ev; // (iteration index, start mark), timing on
     std::vector<cudaEvent_t> ev_pool;
     size_t ev_used = 0;
+
+    PageToucher *toucher = nullptr;                      // result pages, created by the first large fetch
 
     // host compaction of the C route (ExpTM-C as a CPU gather)
     HostPool *pool = nullptr;
@@ -2143,6 +2235,34 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
     return HYTG_OK;
 }
 
+// Start faulting in a result buffer's pages; false if it is too small to be
+// worth waking the threads for or they cannot be made.
+bool touch_start(hytg_ctx *c, void *out, uint64_t bytes) {
+    if (bytes < (4u << 20)) return false;
+    if (!c->toucher) {
+        try {
+            c->toucher = new PageToucher(std::max(1u, std::min(7u, std::thread::hardware_concurrency())));
+        } catch (...) {
+            return false;
+        }
+    }
+    c->toucher->start(out, bytes);
+    return true;
+}
+
+// Copy the last run's result to the caller, whose pages may be present already.
+hytg_status fetch_result(hytg_ctx *c, void *out, uint64_t out_bytes, bool touched) {
+    if (!c->have_result) return fail(c, HYTG_ERR_STATE, "no completed run");
+    const uint64_t need = c->V * 4 * (c->batch_mode != kBatchNone ? c->batch_K : 1);
+    if (out_bytes < need) return fail(c, HYTG_ERR_ARG, "output buffer too small");
+    CK(cudaSetDevice(c->device));
+    if (!touched && touch_start(c, out, need)) c->toucher->finish();
+    CK(cudaMemcpyAsync(out, c->batch_mode != kBatchNone ? c->d_bout : (void *)c->d_out, need,
+                       cudaMemcpyDeviceToHost, c->s_main));
+    CK(cudaStreamSynchronize(c->s_main));
+    return HYTG_OK;
+}
+
 }  // namespace
 
 // ===================================================================== ABI
@@ -2182,16 +2302,20 @@ hytg_status hytg_create(hytg_ctx **out, int device) {
     for (int i = 0; i < 2; ++i) ck(cudaEventCreateWithFlags(&c->ev_cstage[i], cudaEventDisableTiming));
     ck(cudaEventCreateWithFlags(&c->ev_clist, cudaEventDisableTiming));
     for (int i = 0; i < 2; ++i) ck(cudaEventCreate(&c->ev_run[i]));
-    ck(cudaMalloc(&c->d_overflow, sizeof(unsigned int)));
-    ck(cudaMalloc(&c->d_err, sizeof(unsigned int)));
-    ck(cudaMemset(c->d_err, 0, sizeof(unsigned int)));
-    ck(cudaMalloc(&c->d_prsums, 2 * sizeof(double)));
+    ck(cudaMalloc(&c->d_report, sizeof(RunReport)));
+    ck(cudaHostAlloc((void **)&c->h_report, sizeof(RunReport), cudaHostAllocDefault));
+    if (c->d_report) {
+        ck(cudaMemset(c->d_report, 0, sizeof(RunReport)));
+        c->d_overflow = &c->d_report->overflow;
+        c->d_err = &c->d_report->err;
+        c->d_prsums = c->d_report->prsums;
+        c->d_src_work = &c->d_report->src_work;
+        c->d_link_ctr = c->d_report->link_ctr;
+        c->d_sp = c->d_report->sp;
+    }
     ck(cudaMalloc(&c->d_src, 64 * sizeof(unsigned int)));
-    ck(cudaMalloc(&c->d_src_work, sizeof(unsigned long long)));
     ck(cudaMalloc(&c->d_bsums, 64 * sizeof(double)));
     ck(cudaMalloc(&c->d_alive, sizeof(unsigned long long)));
-    ck(cudaMalloc(&c->d_sp, kSpSlots * sizeof(unsigned long long)));
-    ck(cudaMalloc(&c->d_link_ctr, 2 * kRoutes * sizeof(unsigned long long)));
     ck(cudaStreamCreateWithFlags(&c->s_cap, cudaStreamNonBlocking));
     ck(cudaStreamCreateWithFlags(&c->s_cap2, cudaStreamNonBlocking));
     ck(cudaMalloc(&c->d_loop_fh, 1024 * sizeof(unsigned long long)));
@@ -2215,15 +2339,12 @@ hytg_status hytg_destroy(hytg_ctx *c) {
     if (c->s_main) cudaStreamSynchronize(c->s_main);
     free_graph(c);
     dfree(c->d_pool);
-    dfree(c->d_overflow);
-    dfree(c->d_err);
-    dfree(c->d_prsums);
+    dfree(c->d_report);
+    if (c->h_report) cudaFreeHost(c->h_report);
+    delete c->toucher;
     dfree(c->d_src);
-    dfree(c->d_src_work);
     dfree(c->d_bsums);
     dfree(c->d_alive);
-    dfree(c->d_sp);
-    dfree(c->d_link_ctr);
     for (auto e : c->ev_pool) cudaEventDestroy(e);
     for (int i = 0; i < kMaxStreams; ++i) {
         if (c->s_f[i]) cudaStreamDestroy(c->s_f[i]);
@@ -2581,9 +2702,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         if (algo == kSSSP && c->batch_mode == kBatchNone)
             delta = c->sssp_delta < 0 ? c->auto_delta : (uint64_t)c->sssp_delta;
         unsigned int bucket = delta ? (unsigned int)std::min<uint64_t>(delta, 0xFFFFFFFEull) : 0xFFFFFFFFu;
-        CK(cudaMemsetAsync(c->d_err, 0, 4, c->s_main));
-        CK(cudaMemsetAsync(c->d_sp, 0, kSpSlots * 8, c->s_main));
-        CK(cudaMemsetAsync(c->d_link_ctr, 0, 2 * kRoutes * 8, c->s_main));
+        CK(cudaMemsetAsync(c->d_report, 0, sizeof(RunReport), c->s_main));
         c->sp_launches = 0;
         c->timeline.clear();
         if ((algo == kPR || algo == kPPR) && c->d_hub_rep && c->batch_mode == kBatchNone)
@@ -2593,8 +2712,6 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
             ScopedTime t(c, HYTG_K_INIT, c->s_main);
             if (c->batch_mode != kBatchNone) {
                 CK(cudaMemcpyAsync(c->d_src, src_int, sizeof(src_int), cudaMemcpyHostToDevice, c->s_main));
-                CK(cudaMemsetAsync(c->d_src_work, 0, 8, c->s_main));
-                CK(cudaMemsetAsync(c->d_overflow, 0, 4, c->s_main));
                 for (uint32_t g = 0; g * kFrameSources < c->batch_K; ++g)
                     CK(launch_frame_init(c->bs, c->V, g, c->s_main));
                 CK(launch_b_init(c->bs, c->V, c->n_words_alloc, c->d_src, c->batch_K,
@@ -2684,20 +2801,9 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
             else
                 CK(launch_to_original(st.perm, c->d_val, c->d_out, c->V, c->s_main));
         }
-        unsigned int ovf = 0, ierr = 0;
-        double prs[2] = {0, 0};
-        CK(cudaMemcpyAsync(&ovf, c->d_overflow, 4, cudaMemcpyDeviceToHost, c->s_main));
-        CK(cudaMemcpyAsync(&ierr, c->d_err, 4, cudaMemcpyDeviceToHost, c->s_main));
-        if ((algo == kPR || algo == kPPR) && c->batch_mode == kBatchNone)
-            CK(cudaMemcpyAsync(prs, c->d_prsums, 16, cudaMemcpyDeviceToHost, c->s_main));
-        unsigned long long swork = 0, extra = 0;
         const uint32_t n_sp = std::min<uint32_t>(c->sp_launches + 1, kSpSlots);
-        std::vector<unsigned long long> sp(n_sp, 0);
-        unsigned long long lctr[2 * kRoutes] = {};
-        CK(cudaMemcpyAsync(sp.data(), c->d_sp, n_sp * 8, cudaMemcpyDeviceToHost, c->s_main));
-        CK(cudaMemcpyAsync(lctr, c->d_link_ctr, sizeof lctr, cudaMemcpyDeviceToHost, c->s_main));
-        if (c->batch_mode != kBatchNone)
-            CK(cudaMemcpyAsync(&swork, c->d_src_work, 8, cudaMemcpyDeviceToHost, c->s_main));
+        CK(cudaMemcpyAsync(c->h_report, c->d_report, offsetof(RunReport, sp) + n_sp * 8, cudaMemcpyDeviceToHost,
+                           c->s_main));
         CK(cudaEventRecord(c->ev_run[1], c->s_main));
         CK(cudaStreamSynchronize(c->s_main));
         CK(cudaGetLastError());
@@ -2708,10 +2814,16 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
             c->stats.device_ms = dms;
         }
         c->stats.wall_ms = std::chrono::duration<double, std::milli>(t_end - t_start).count();
-        c->stats.pr_rank_sum = prs[0];
-        c->stats.pr_residual_sum = prs[1];
+        const RunReport &rep = *c->h_report;
+        const unsigned int ovf = rep.overflow, ierr = rep.err;
+        const unsigned long long *sp = rep.sp, *lctr = rep.link_ctr;
+        unsigned long long extra = 0;
+        if ((algo == kPR || algo == kPPR) && c->batch_mode == kBatchNone) {
+            c->stats.pr_rank_sum = rep.prsums[0];
+            c->stats.pr_residual_sum = rep.prsums[1];
+        }
         c->stats.n_sources = c->batch_K;
-        for (unsigned long long x : sp) extra += x;
+        for (uint32_t k = 0; k < n_sp; ++k) extra += sp[k];
         c->stats.extra_edges = extra;
         for (int r = 0; r < kRoutes; ++r) {
             c->stats.link_sector_bytes[r] = lctr[2 * r] * 32ull;
@@ -2721,7 +2833,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         c->stats.link_sector_bytes[kRouteF] = c->stats.link_line_bytes[kRouteF] = c->stats.link_bytes[kRouteF];
         if (c->compact_host > 0)
             c->stats.link_sector_bytes[kRouteC] = c->stats.link_line_bytes[kRouteC] = c->stats.link_bytes[kRouteC];
-        c->stats.source_edges = c->batch_mode != kBatchNone ? swork : c->stats.edges_relaxed;
+        c->stats.source_edges = c->batch_mode != kBatchNone ? rep.src_work : c->stats.edges_relaxed;
         for (size_t i = 0; i + 1 < c->iter_ev.size(); ++i) {
             // host-issued iterations only: a mark and the next iteration's mark
             const size_t k = c->iter_ev[i].first;
@@ -2782,8 +2894,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
             r.part_first = tl.part_first;
             r.part_last = tl.part_last;
             if (tl.sp_slot >= 0)
-                r.edges = (uint32_t)tl.sp_slot < kSpSlots - 1 && (size_t)tl.sp_slot < sp.size() ? sp[tl.sp_slot]
-                                                                                            : UINT64_MAX;
+                r.edges = (uint32_t)tl.sp_slot < kSpSlots - 1 && (uint32_t)tl.sp_slot < n_sp ? sp[tl.sp_slot] : UINT64_MAX;
             c->timeline.push_back(r);
         }
         for (auto &tl : c->timed) {
@@ -2875,9 +2986,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     s = ensure_cache(c, n_arrays);
     if (s == HYTG_OK) s = ensure_second_pass(c, algo);
     if (s != HYTG_OK) return s;
-    CK(cudaMemsetAsync(c->d_err, 0, 4, c->s_main));
-    CK(cudaMemsetAsync(c->d_overflow, 0, 4, c->s_main));
-    CK(cudaMemsetAsync(c->d_src_work, 0, 8, c->s_main));
+    CK(cudaMemsetAsync(c->d_report, 0, offsetof(RunReport, sp), c->s_main));
     CK(launch_b_init(c->bs, c->V, c->n_words_alloc, c->d_src, 0, 0.0f, c->d_bm[0], c->s_main));
     c->serving = true;
     c->serve_algo = algo;
@@ -2955,10 +3064,9 @@ hytg_status hytg_serve_fetch(hytg_ctx *c, uint32_t slot, void *out, uint64_t out
     CK(launch_serve_extract(c->bs, c->V, slot, c->d_perm, c->serve_admit_it[slot], c->d_bout,
                             c->d_bsums, c->s_main));
     CK(cudaMemcpyAsync(out, c->d_bout, c->V * 4, cudaMemcpyDeviceToHost, c->s_main));
-    unsigned int ovf = 0, ierr = 0;
-    CK(cudaMemcpyAsync(&ovf, c->d_overflow, 4, cudaMemcpyDeviceToHost, c->s_main));
-    CK(cudaMemcpyAsync(&ierr, c->d_err, 4, cudaMemcpyDeviceToHost, c->s_main));
+    CK(cudaMemcpyAsync(c->h_report, c->d_report, offsetof(RunReport, prsums), cudaMemcpyDeviceToHost, c->s_main));
     CK(cudaStreamSynchronize(c->s_main));
+    const unsigned int ovf = c->h_report->overflow, ierr = c->h_report->err;
     c->serve_busy &= ~bit;
     release_idle_frame(c, slot / kFrameSources);
     if (ierr) return fail(c, HYTG_ERR_CUDA, "internal index check failed");
@@ -2994,14 +3102,20 @@ hytg_status hytg_serve_get_info(hytg_ctx *c, hytg_serve_info *out) {
 
 hytg_status hytg_fetch_result(hytg_ctx *c, void *out, uint64_t out_bytes) {
     if (!c || !out) return HYTG_ERR_ARG;
-    if (!c->have_result) return fail(c, HYTG_ERR_STATE, "no completed run");
-    const uint64_t need = c->V * 4 * (c->batch_mode != kBatchNone ? c->batch_K : 1);
-    if (out_bytes < need) return fail(c, HYTG_ERR_ARG, "output buffer too small");
-    CK(cudaSetDevice(c->device));
-    CK(cudaMemcpyAsync(out, c->batch_mode != kBatchNone ? c->d_bout : (void *)c->d_out, need,
-                       cudaMemcpyDeviceToHost, c->s_main));
-    CK(cudaStreamSynchronize(c->s_main));
-    return HYTG_OK;
+    return fetch_result(c, out, out_bytes, false);
+}
+
+hytg_status hytg_run_fetch(hytg_ctx *c, hytg_algo algo, const uint32_t *sources, uint32_t n_sources, void *out,
+                           uint64_t out_bytes) {
+    if (!c || !out) return HYTG_ERR_ARG;
+    // whatever the run returns, the threads are done with the buffer before
+    // this call is
+    const uint64_t rows = algo == HYTG_CC || algo == HYTG_PAGERANK ? 1 : n_sources;
+    const uint64_t need = c->loaded ? c->V * 4 * rows : 0;
+    const bool touching = touch_start(c, out, std::min(out_bytes, need));
+    const hytg_status s = hytg_run(c, algo, sources, n_sources);
+    if (touching) c->toucher->finish();
+    return s == HYTG_OK ? fetch_result(c, out, out_bytes, touching) : s;
 }
 
 hytg_status hytg_fetch_pagerank_state(hytg_ctx *c, float *rank, float *delta, uint64_t V) {

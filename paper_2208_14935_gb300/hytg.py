@@ -105,6 +105,7 @@ def load(path: Optional[str] = None):
             "hytg_get_param": [vp, ctypes.c_char_p, P(dbl)],
             "hytg_run": [vp, i32, vp, u32],
             "hytg_fetch_result": [vp, vp, u64],
+            "hytg_run_fetch": [vp, i32, vp, u32, vp, u64],
             "hytg_fetch_pagerank_state": [vp, vp, vp, u64],
             "hytg_get_stats": [vp, P(hytg_stats)],
             "hytg_get_info": [vp, P(hytg_info)],
@@ -193,6 +194,16 @@ def hytg_fetch_result(ctx, V: int, algo: int, n_sources: int = 1) -> np.ndarray:
     out = np.empty(V * n_sources, dtype=dt)
     _check(ctx, load().hytg_fetch_result(ctx, _ptr(out), out.nbytes))
     return out if n_sources == 1 else out.reshape(n_sources, V)
+
+
+def hytg_run_fetch(ctx, V: int, algo: int, sources: Optional[Sequence[int]] = None) -> np.ndarray:
+    """hytg_run and hytg_fetch_result in one call, the result's pages faulted
+    in while the run is on the device."""
+    src = None if sources is None else np.ascontiguousarray(sources, np.uint32)
+    n = 0 if src is None else len(src)
+    out = np.empty(V * max(1, n), dtype=np.float32 if algo in (HYTG_PAGERANK, HYTG_PPR) else np.uint32)
+    _check(ctx, load().hytg_run_fetch(ctx, int(algo), _ptr(src), n, _ptr(out), out.nbytes))
+    return out if n <= 1 else out.reshape(n, V)
 
 
 def hytg_fetch_pagerank_state(ctx, V: int):
@@ -398,14 +409,13 @@ class Engine:
         whose result has one row per source)."""
         a = ALGOS[algo] if isinstance(algo, str) else int(algo)
         if source is None:
-            hytg_run(self.ctx, a, None)
-            return hytg_fetch_result(self.ctx, self.V, a)
-        if np.ndim(source) == 0:
-            hytg_run(self.ctx, a, [int(source)])
-            return hytg_fetch_result(self.ctx, self.V, a)
-        srcs = [int(x) for x in source]
-        hytg_run(self.ctx, a, srcs)
-        return hytg_fetch_result(self.ctx, self.V, a, len(srcs))
+            srcs = None
+        else:
+            srcs = [int(source)] if np.ndim(source) == 0 else [int(x) for x in source]
+        if self.V and (srcs is None or 1 <= len(srcs) <= 64):
+            return hytg_run_fetch(self.ctx, self.V, a, srcs)
+        hytg_run(self.ctx, a, srcs)                # no graph, or a number of sources it refuses
+        return hytg_fetch_result(self.ctx, self.V, a, 1 if srcs is None else len(srcs))
 
     def stats(self) -> Dict:
         return hytg_get_stats(self.ctx)
