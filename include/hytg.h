@@ -238,7 +238,8 @@ hytg_status hytg_set_device_budget(hytg_ctx *ctx, uint64_t bytes);
  * edges, no F route and at most 1,024 partitions run several at a time in one
  * kernel of the body, the C route's lists read from mapped host memory there
  * unless "compact_host" is on),
- * while batched runs keep F and C iterations in the graph too: one IF node
+ * while batched runs (PPR: of graphs up to 2^20 edges) keep F and C
+ * iterations in the graph too: one IF node
  * per partition copies it into a staging slot and relaxes it, one IF node
  * gathers and relaxes the C route, each F copy moves one partition (no task
  * combination, partition order), and only a C route larger than the

@@ -213,13 +213,16 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
     LinkCount lc;
     walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
         unsigned int dv[kBatchSteps];
-        unsigned long long vis[kBatchSteps];
+        unsigned long long seen[kBatchSteps];
         load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
+        // reached before, or marked by another edge of this iteration: a hub's
+        // word would otherwise take an atomic from every edge that ends there
 #pragma unroll
-        for (int q = 0; q < kBatchSteps; ++q) vis[q] = ed[q].ok ? __ldcg(&b.vis[dv[q]]) : ~0ull;
+        for (int q = 0; q < kBatchSteps; ++q)
+            seen[q] = ed[q].ok ? __ldcg(&b.vis[dv[q]]) | __ldcg(&b.nxt[dv[q]]) : ~0ull;
 #pragma unroll
         for (int q = 0; q < kBatchSteps; ++q) {
-            const unsigned long long nb = ed[q].pay & ~vis[q];
+            const unsigned long long nb = ed[q].pay & ~seen[q];
             if (ed[q].ok && nb) atomicOr(&b.nxt[dv[q]], nb);
         }
     });
@@ -228,8 +231,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
 
 // Multi-source SSSP and batched PPR relax.  A warp loads 32 edges at once
 // (coalesced), one per lane, each with its source vertex u and the mask of
-// sources active at u.  PPR: every lane pushes its own edge, a frame of 8
-// seeds per pair of vector reductions (ppr_push_vec).  SSSP: when the masks
+// sources active at u.  PPR: ppr_edges.  SSSP: when the masks
 // are dense (on average "batch_sparse_below" or more sources per edge) the
 // warp walks its edges one at a time with a lane per source (s = lane and
 // lane + 32), reading each source's value row in one sector per frame;
@@ -284,6 +286,50 @@ __device__ __forceinline__ void mssssp_edges(const BatchState &b, unsigned int v
     }
 }
 
+// PPR push of 32 edges, one per lane: u's messages for the seeds in m to w's
+// residuals.  Eight lanes share an edge, each with four seeds (a 16-byte half
+// of a frame's sector), so a warp has four edges in flight per load and per
+// vector reduction; a lane that walked its own edge's eight halves waited for
+// each load in turn.  The other seeds of a half carry a zero message (the take
+// kernels write 0 for every seed they do not take), so adding them leaves
+// their residuals unchanged; a half with no active seed is skipped.
+//
+// w's frontier bit is looked at before it is set: with R-MAT's in-degree skew
+// 15 % of the edges of a 2^18-vertex graph end in the first 32 vertices, one
+// word, and as many atomics on one address took most of the relax's time.
+// Both together: 590 K edges with 32 seeds each, 260 -> 70 us (70 G vector
+// reductions/s); replica frames for the hub ids, as single-source PageRank has,
+// gained nothing after this and hid the hubs' residuals from the second passes
+// (183 iterations instead of 103 on R-MAT 18).
+// (The plain load may miss a bit set meanwhile, never see one too many: bits
+// are only cleared between relaxes, by earlier kernels of the main stream.)
+__device__ __forceinline__ void ppr_edges(const BatchState &b, unsigned int w, unsigned int u, unsigned int m,
+                                          unsigned int *bm) {
+    const int lane = threadIdx.x & 31, part = lane & 7, sub = lane >> 3;
+    if (m && !((bm[w >> 5] >> (w & 31)) & 1u)) atomicOr(&bm[w >> 5], 1u << (w & 31));
+    constexpr int kTurns = 4;                       // 16 edges' messages in flight
+#pragma unroll
+    for (int i0 = 0; i0 < 8; i0 += kTurns) {
+        float4 x[kTurns];
+        float *to[kTurns];
+#pragma unroll
+        for (int i = 0; i < kTurns; ++i) {
+            const int e = (i0 + i) * 4 + sub;
+            const unsigned int we = __shfl_sync(0xffffffffu, w, e), ue = __shfl_sync(0xffffffffu, u, e);
+            const unsigned int me = __shfl_sync(0xffffffffu, m, e);
+            to[i] = nullptr;
+            if ((me >> (4 * part)) & 0xFu) {
+                const unsigned int g = part >> 1, h = 4 * (part & 1);
+                x[i] = __ldcg((const float4 *)(b.msg[g] + (unsigned long long)ue * kFrameSources + h));
+                to[i] = b.delta[g] + (unsigned long long)we * kFrameSources + h;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kTurns; ++i)
+            if (to[i]) atomicAdd((float4 *)to[i], x[i]);
+    }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, ListArrays la,
                                                               const Summary *sum, RelaxTask t,
@@ -301,15 +347,9 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, List
 #pragma unroll
         for (int q = 0; q < kBatchSteps; ++q) {
             const unsigned long long f = ed[q].ok ? ed[q].pay : 0ull;
-            if (MODE == kBatchPPR) {
-                // a lane per edge, a frame's 8 seeds per pair of vector reductions
-                if (f) {
-                    atomicOr(&bm[dv[q] >> 5], 1u << (dv[q] & 31));
-                    ppr_push_vec(b, ed[q].vid, dv[q], (unsigned int)f);
-                }
-            } else {
-                if (__any_sync(0xffffffffu, f != 0)) mssssp_edges(b, dv[q], wv[q], ed[q].vid, f, overflow);
-            }
+            if (!__any_sync(0xffffffffu, f != 0)) continue;
+            if (MODE == kBatchPPR) ppr_edges(b, dv[q], ed[q].vid, (unsigned int)f, bm);
+            else mssssp_edges(b, dv[q], wv[q], ed[q].vid, f, overflow);
         }
     });
     flush_link(lc, t.link_ctr);

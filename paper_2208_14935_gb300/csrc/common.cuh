@@ -239,25 +239,6 @@ __device__ __forceinline__ float *brank(const BatchState &b, unsigned long long 
 __device__ __forceinline__ float *bmsg(const BatchState &b, unsigned long long v, unsigned int s) {
     return b.msg[s >> 3] + v * kFrameSources + (s & 7);
 }
-// PPR push of u's messages along one edge u -> w for the seeds in `m` (a
-// 32-bit mask): per frame holding an active seed, the frame's 8 messages of
-// u are read as two float4 and added to w's 8 residuals with two vector
-// reductions (red.global.add.v4.f32, one L2 operation for four seeds); a
-// half with no active seed is skipped.  The other seeds of a half carry a
-// zero message (the take kernels write 0 for every seed they do not take),
-// so adding them leaves their residuals unchanged.
-__device__ __forceinline__ void ppr_push_vec(const BatchState &b, unsigned long long u, unsigned long long w,
-                                             unsigned int m) {
-    while (m) {
-        const unsigned int g = (unsigned int)(__ffs(m) - 1) >> 3;
-        const unsigned int fm = (m >> (8 * g)) & 0xFFu;
-        m &= ~(0xFFu << (8 * g));
-        const float4 *src = (const float4 *)(b.msg[g] + u * kFrameSources);
-        float4 *dst = (float4 *)(b.delta[g] + w * kFrameSources);
-        if (fm & 0x0Fu) atomicAdd(dst, __ldcg(src));
-        if (fm & 0xF0u) atomicAdd(dst + 1, __ldcg(src + 1));
-    }
-}
 constexpr unsigned int kHubReplicas = 256;
 
 // log2 of a power of two, else -1.

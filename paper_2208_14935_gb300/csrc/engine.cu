@@ -1421,11 +1421,22 @@ bool loop_applies(const hytg_ctx *c) {
 }
 
 // F and C iterations can stay in the device loop: batched runs at "device_loop"
-// 1, every run at 2; not with host compaction, forced random routes, more
+// 1 (PPR: of graphs up to kLoopFcEdges edges), every run at 2; not with host compaction, forced random routes, more
 // partitions than 1024 IF nodes, or a staging slot without room for one
 // partition.
+//
+// A partition's IF node costs about 1 us per iteration closed and 20 to 40 us
+// open, copies one partition at a time and shares one chain of launches per
+// slot; the host combines partitions into tasks and overlaps them on several
+// streams.  A 32-seed PPR has about a hundred F iterations: in the loop against
+// from the host, R-MAT 16 44 / 30 ms, R-MAT 18 78 / 47 ms, R-MAT 20 194 / 156 ms.
+// Batched BFS and SSSP have two or three, and their option promises the loop
+// (R-MAT 20 3.0 against 2.4 ms), as it does for small PPR.
+constexpr uint64_t kLoopFcEdges = 1u << 20;
 bool loop_fc_wanted(const hytg_ctx *c) {
-    if (c->device_loop < 2 && c->batch_mode == kBatchNone) return false;
+    if (c->device_loop < 2 &&
+        (c->batch_mode == kBatchNone || (c->batch_mode == kBatchPPR && c->E > kLoopFcEdges)))
+        return false;
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
     return c->compact_host == 0 && c->force_route != 5 && N >= 1 && N <= 1024 && c->carve.n_slots >= 1 &&
            c->carve.slot_edges >= c->max_part_edges;
