@@ -211,10 +211,10 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_msbfs(BatchState b, ListA
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     LinkCount lc;
-    walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
+    walk_task<kBatchSteps, true, false>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
         unsigned int dv[kBatchSteps];
         unsigned long long seen[kBatchSteps];
-        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
+        load_entries<false>(t.src.dst, t.src.dst_bits, ed, dv);
         // reached before, or marked by another edge of this iteration: a hub's
         // word would otherwise take an atomic from every edge that ends there
 #pragma unroll
@@ -339,11 +339,10 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_mswarp(BatchState b, List
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     LinkCount lc;
-    lc.weights = MODE == kBatchSSSP;
-    walk_task<kBatchSteps, true>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
+    walk_task<kBatchSteps, true, MODE == kBatchSSSP>(la, rv, t, kb, ke, lc, [&](const Edge<true> (&ed)[kBatchSteps], unsigned long long) {
         unsigned int dv[kBatchSteps], wv[kBatchSteps] = {};
-        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
-        if (MODE == kBatchSSSP) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
+        load_entries<false>(t.src.dst, t.src.dst_bits, ed, dv);
+        if (MODE == kBatchSSSP) load_entries<true>(t.src.w, t.src.w_bits, ed, wv);
 #pragma unroll
         for (int q = 0; q < kBatchSteps; ++q) {
             const unsigned long long f = ed[q].ok ? ed[q].pay : 0ull;

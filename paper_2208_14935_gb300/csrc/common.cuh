@@ -201,7 +201,10 @@ struct AlgoState {
     const unsigned long long *b_fr;   // BFS/SSSP: 64-bit source mask per vertex
     const unsigned int *b_fr32;       // PPR: 32-bit seed mask per vertex
     unsigned long long *src_work;     // sum over entries of popcount(mask) * degree
+    unsigned long long V;
 };
+// Edges from which a PageRank relax sums hub ids in shared memory (rank_ids).
+constexpr unsigned long long kRankNarrow = 1ull << 14, kRankWide = 1ull << 23;
 
 enum BatchMode : int { kBatchNone = 0, kBatchBFS = 1, kBatchSSSP = 2, kBatchPPR = 3 };
 

@@ -82,7 +82,6 @@ __device__ __forceinline__ RouteView task_view(RelaxTask &t, const Summary *sum,
 // counts, added once per warp.
 struct LinkCount {
     unsigned int sec = 0, ln = 0;
-    bool weights = false;               // the weight array is read too
 };
 __device__ __forceinline__ void count_link(LinkCount &lc, long long e, long long prev, unsigned int bits) {
     const unsigned long long a = (unsigned long long)e * bits, z = a + bits - 1;
@@ -99,18 +98,19 @@ __device__ __forceinline__ void flush_link(const LinkCount &lc, unsigned long lo
     }
 }
 
-// One edge of a step: its CSR index (compacted buffer: its place in the
-// route), whether the next lane holds the edge after it, and its owner's
-// payload.  BATCH: the owner's per-source word and vertex instead of a value.
+// One edge of a step: the bit positions of its entries in the task's arrays
+// (the weights' only if they are read), whether the next lane holds the edge
+// after it, and its owner's payload.  BATCH: the owner's per-source word and
+// vertex instead of a value.
 template <bool BATCH> struct Edge;
 template <> struct Edge<false> {
     bool ok, adj;
-    long long e;
+    long long dbit, wbit;
     unsigned int pay;
 };
 template <> struct Edge<true> {
     bool ok, adj;
-    long long e;
+    long long dbit, wbit;
     unsigned long long pay;
     unsigned int vid;
 };
@@ -119,25 +119,24 @@ template <> struct Edge<true> {
 // that runs into the next word takes that word from the next lane when that
 // lane holds the next edge (its entry then starts in that word), so a list's
 // words are loaded once; only a list's or a step's last edge may load a second
-// word.  Needs all 32 lanes.
-template <int S, class E>
-__device__ __forceinline__ void load_entries(const unsigned int *p, unsigned int bits, long long off,
-                                             const E (&ed)[S], unsigned int (&out)[S]) {
+// word, beside the first one's load.  Needs all 32 lanes.
+template <bool WEIGHTS, int S, class E>
+__device__ __forceinline__ void load_entries(const unsigned int *p, unsigned int bits, const E (&ed)[S],
+                                             unsigned int (&out)[S]) {
     const unsigned int mask = 0xffffffffu >> (32 - bits);
     unsigned int lo[S], hi[S], sh[S];
 #pragma unroll
     for (int q = 0; q < S; ++q) {
-        const long long bit = ed[q].ok ? ed[q].e * (long long)bits - off : 0;
+        const long long bit = WEIGHTS ? ed[q].wbit : ed[q].dbit;
         const unsigned int *at = p + (bit >> 5);
         sh[q] = (unsigned int)bit & 31u;
         lo[q] = ed[q].ok ? __ldg(at) : 0u;
-        // beside the first word's load, not behind it
         hi[q] = ed[q].ok && !ed[q].adj && sh[q] + bits > 32 ? __ldg(at + 1) : 0u;
     }
 #pragma unroll
     for (int q = 0; q < S; ++q) {
         const unsigned int next = __shfl_down_sync(0xffffffffu, lo[q], 1);
-        out[q] = ed[q].ok ? __funnelshift_r(lo[q], ed[q].adj ? next : hi[q], sh[q]) & mask : 0u;
+        out[q] = __funnelshift_r(lo[q], ed[q].adj ? next : hi[q], sh[q]) & mask;
     }
 }
 
@@ -154,7 +153,7 @@ __device__ __forceinline__ int run_shift(unsigned long long total, unsigned long
 // steps of 32 edges at a time: f(ed, k) gets the lane's S edges and the route
 // edge of the first, its others being 32 apart.  An inconsistent list is
 // recorded in la.err and skipped.
-template <int S, bool BATCH, class F>
+template <int S, bool BATCH, bool WEIGHTS, class F>
 __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &rv, const RelaxTask &t,
                                          unsigned long long run, int sh, unsigned long long kb,
                                          unsigned long long ke, LinkCount &lc, F &&f) {
@@ -225,6 +224,23 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
                 e_prev = (long long)(k0 - 1) + ((long long)la.soff[j] - (long long)la.ebase[j]);
             }
         }
+        // per list, once a window: where its entries lie (for route edge k0, had
+        // it been the list's), and that its edges of this run are present
+        const long long dbase = (delta + (long long)k0) * t.src.dst_bits - t.src.dst_off;
+        const long long wbase = WEIGHTS ? (delta + (long long)k0) * t.src.w_bits - t.src.w_off : 0;
+        {
+            const int next = __shfl_down_sync(0xffffffffu, rel, 1);
+            const int f = rel < 0 ? 0 : rel, z = next < n ? next : n;
+            const long long e0 = delta + (long long)k0;
+            if (__any_sync(0xffffffffu, lane < 31 && f < z &&
+                                            (e0 + f < (long long)t.src.e_lo || e0 + z > (long long)t.src.e_hi))) {
+                if (lane == 0) atomicOr(la.err, 8u);
+                pos = wend;
+                i += 31;
+                continue;
+            }
+        }
+        int before = __popc(__ballot_sync(0xffffffffu, rel < pos));
         for (int b0 = pos; b0 < wend; b0 += 32 * S) {
             Edge<BATCH> ed[S];
 #pragma unroll
@@ -232,11 +248,13 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
                 const int b = b0 + 32 * q;
                 ed[q].ok = ed[q].adj = false;
                 if (b >= wend) continue;            // warp-uniform
-                const int before = __popc(__ballot_sync(0xffffffffu, rel < b));
-                const unsigned int heads =
-                    __reduce_or_sync(0xffffffffu, rel >= b && rel < b + 32 ? 1u << (rel - b) : 0u);
+                const unsigned int at = (unsigned int)(rel - b);
+                const unsigned int heads = __reduce_or_sync(0xffffffffu, at < 32u ? 1u << at : 0u);
                 const int own = before + __popc(heads & (0xffffffffu >> (31 - lane))) - 1;
-                ed[q].e = (long long)(k0 + b + lane) + __shfl_sync(0xffffffffu, delta, own);
+                before += __popc(heads);
+                ed[q].dbit = __shfl_sync(0xffffffffu, dbase, own) + (unsigned int)(b + lane) * t.src.dst_bits;
+                if (WEIGHTS)
+                    ed[q].wbit = __shfl_sync(0xffffffffu, wbase, own) + (unsigned int)(b + lane) * t.src.w_bits;
                 if constexpr (BATCH) {
                     ed[q].pay = __shfl_sync(0xffffffffu, pay64, own);
                     ed[q].vid = __shfl_sync(0xffffffffu, vid, own);
@@ -246,17 +264,14 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
                 ed[q].ok = b + lane < wend;
                 ed[q].adj = lane < 31 && b + lane + 1 < wend && !((heads >> (lane + 1)) & 1u);
                 if (t.link_ctr) {
-                    long long p = __shfl_up_sync(0xffffffffu, ed[q].e, 1);
+                    const long long e = (long long)(k0 + b + lane) + __shfl_sync(0xffffffffu, delta, own);
+                    long long p = __shfl_up_sync(0xffffffffu, e, 1);
                     if (lane == 0) p = e_prev;
                     if (ed[q].ok) {
-                        count_link(lc, ed[q].e, p, t.src.dst_bits);
-                        if (lc.weights) count_link(lc, ed[q].e, p, t.src.w_bits);
+                        count_link(lc, e, p, t.src.dst_bits);
+                        if (WEIGHTS) count_link(lc, e, p, t.src.w_bits);
                     }
-                    e_prev = __shfl_sync(0xffffffffu, ed[q].e, min(31, wend - 1 - b));
-                }
-                if (ed[q].ok && (ed[q].e < (long long)t.src.e_lo || ed[q].e >= (long long)t.src.e_hi)) {
-                    atomicOr(la.err, 8u);
-                    ed[q].ok = ed[q].adj = false;
+                    e_prev = __shfl_sync(0xffffffffu, e, min(31, wend - 1 - b));
                 }
             }
             f(ed, k0 + b0 + lane);
@@ -267,7 +282,7 @@ __device__ __forceinline__ void walk_run(const ListArrays &la, const RouteView &
 }
 
 // Every run of the task, one per warp in turn.
-template <int S, bool BATCH, class F>
+template <int S, bool BATCH, bool WEIGHTS, class F>
 __device__ __forceinline__ void walk_task(const ListArrays &la, const RouteView &rv, const RelaxTask &t,
                                           unsigned long long kb, unsigned long long ke, LinkCount &lc, F &&f) {
     if (kb >= ke) return;
@@ -276,7 +291,7 @@ __device__ __forceinline__ void walk_task(const ListArrays &la, const RouteView 
     const unsigned long long last = (ke - 1) >> sh;
     for (unsigned long long run = (kb >> sh) + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); run <= last;
          run += nwarps)
-        walk_run<S, BATCH>(la, rv, t, run, sh, kb, ke, lc, f);
+        walk_run<S, BATCH, WEIGHTS>(la, rv, t, run, sh, kb, ke, lc, f);
 }
 
 // Place a block's list entries: every thread of the block calls it, each warp

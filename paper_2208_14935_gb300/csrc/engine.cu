@@ -1078,6 +1078,7 @@ AlgoState algo_state(hytg_ctx *c, int algo, unsigned int bucket_limit = 0xFFFFFF
     st.n_hub_rep = pr && c->d_hub_rep ? c->n_hub_rep : 0;
     st.prio = pr && c->priority != 0 && c->batch_mode == kBatchNone;
     st.loop = nullptr;
+    st.V = c->V;
     return st;
 }
 

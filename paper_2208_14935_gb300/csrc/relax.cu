@@ -64,8 +64,8 @@ __device__ __forceinline__ void relax_edges(const AlgoState &st, const RelaxTask
                                             const Edge<false> (&ed)[kSteps], float *hub_rep) {
     constexpr bool rank = ALGO == kPR || ALGO == kPPR;
     unsigned int dv[kSteps], wv[kSteps] = {}, cur[kSteps];
-    load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
-    if (ALGO == kSSSP) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
+    load_entries<false>(t.src.dst, t.src.dst_bits, ed, dv);
+    if (ALGO == kSSSP) load_entries<true>(t.src.w, t.src.w_bits, ed, wv);
     if (!rank) {
         // the values are read together before any reduction is issued (a
         // reduction between them would make the loads wait for one another)
@@ -78,18 +78,90 @@ __device__ __forceinline__ void relax_edges(const AlgoState &st, const RelaxTask
 }
 
 template <int ALGO>
-__global__ void __launch_bounds__(kRelaxBlock) k_relax(AlgoState st, ListArrays la,
+__global__ void __launch_bounds__(kRelaxBlock, 3) k_relax(AlgoState st, ListArrays la,
                                                        const Summary *sum, RelaxTask t) {
     if (st.loop && !st.loop->work) return;
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     float *hub_rep = st.hub_rep ? st.hub_rep + (size_t)(sm_id() % kHubReplicas) * st.n_hub_rep : nullptr;
     LinkCount lc;
-    lc.weights = ALGO == kSSSP;
-    walk_task<kSteps, false>(la, rv, t, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long) {
+    walk_task<kSteps, false, ALGO == kSSSP>(la, rv, t, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long) {
         relax_edges<ALGO>(st, t, ed, hub_rep);
     });
     flush_link(lc, t.link_ctr);
+}
+
+// PageRank and PPR pushes with the hottest targets summed on chip.  What bounds
+// these relaxes is the rate of L2 reductions: 190 G/s to spread-out addresses,
+// 140 to 165 with R-MAT's in-degree skew and per-SM replicas of 4,096 hub ids.
+// Hub sorting puts the hottest targets at the lowest ids, so a block of 1,024
+// threads (one per SM) sums the pushes to ids below ns in shared memory and adds
+// the sums to delta at its end, four ids per vector reduction; a probe with the
+// skew of 2^20 / 2^24 vertices then runs at 261 / 221 G pushes/s (ns = 16,384)
+// against 137 / 166 with the replicas, and the relax of R-MAT 24's cache, 157 M
+// edges, at 240 G pushes/s against 94.  delta also holds the hubs' residuals
+// once the launch ends, where a second pass finds them (replicas are folded
+// once per iteration): R-MAT 20, resident, 71 iterations instead of 97.  Whole
+// runs: 22.5 -> 15 ms there, PPR on R-MAT 24 238 -> 210 ms.  TB: a second,
+// device-sized task in the same launch.
+//
+// The kRankHot hottest ids have a sum per lane: an addition to shared memory is
+// a compare-and-swap loop, and where a few vertices take a large share of the
+// edges (Chung-Lu: 22 % end in 64 of 2^18) the lanes of a warp that meet in one
+// word repeat it once each (a PageRank there: 18.8 ms, 9.3 with the replicas).
+constexpr int kRankHot = 64;
+inline unsigned int rank_smem(unsigned int ns) { return (ns + kRankHot * 32) * 4; }
+__device__ __forceinline__ void rank_edges(const AlgoState &st, const RelaxTask &t, const Edge<false> (&ed)[kSteps],
+                                           float *acc, unsigned int ns) {
+    unsigned int dv[kSteps];
+    load_entries<false>(t.src.dst, t.src.dst_bits, ed, dv);
+#pragma unroll
+    for (int q = 0; q < kSteps; ++q) {
+        if (!ed[q].ok) continue;
+        const float x = __uint_as_float(ed[q].pay);
+        if (dv[q] < kRankHot) atomicAdd(&acc[ns + dv[q] * 32 + (threadIdx.x & 31)], x);
+        else if (dv[q] < ns) atomicAdd(&acc[dv[q]], x);
+        else atomicAdd(&st.delta[dv[q]], x);
+    }
+}
+
+template <int BLOCK, bool TB>
+__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_relax_rank(AlgoState st, ListArrays la, const Summary *sum,
+                                                                    RelaxTask ta, RelaxTask tb, unsigned int ns) {
+    extern __shared__ float4 acc4[];
+    if (st.loop && !st.loop->work) return;
+    float *acc = reinterpret_cast<float *>(acc4);
+    unsigned long long kb, ke, zb = 0, eb = 0;
+    const RouteView va = task_view(ta, sum, kb, ke);
+    RouteView vb{};
+    if (TB) vb = task_view(tb, sum, zb, eb);
+    if (kb >= ke && zb >= eb) return;
+    for (unsigned int i = threadIdx.x; i < (ns + kRankHot * 32) / 4; i += BLOCK) acc4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    LinkCount lc, lb;
+    walk_task<kSteps, false, false>(la, va, ta, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long) {
+        rank_edges(st, ta, ed, acc, ns);
+    });
+    flush_link(lc, ta.link_ctr);
+    if (TB) {
+        walk_task<kSteps, false, false>(la, vb, tb, zb, eb, lb, [&](const Edge<false> (&ed)[kSteps], unsigned long long) {
+            rank_edges(st, tb, ed, acc, ns);
+        });
+        flush_link(lb, tb.link_ctr);
+    }
+    __syncthreads();
+    for (int v = threadIdx.x >> 5; v < kRankHot; v += BLOCK / 32) {
+        float x = acc[ns + v * 32 + (threadIdx.x & 31)];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0) acc[v] = x;    // ids below kRankHot have no other sum
+    }
+    __syncthreads();
+    for (unsigned int i = threadIdx.x; i < ns / 4; i += BLOCK) {
+        const float4 x = acc4[i];
+        if (x.x != 0.f || x.y != 0.f || x.z != 0.f || x.w != 0.f)
+            atomicAdd(reinterpret_cast<float4 *>(st.delta) + i, x);
+    }
 }
 
 // Two device-sized routes in one launch (cache and zero-copy in the device
@@ -108,20 +180,20 @@ __global__ void __launch_bounds__(kRelaxBlock) k_relax_pair(AlgoState st, ListAr
     const int sh = run_shift(ea + eb, nwarps);
     const unsigned long long na = (ea + (1ull << sh) - 1) >> sh, nb = (eb + (1ull << sh) - 1) >> sh;
     LinkCount la_ct, lb_ct;
-    la_ct.weights = lb_ct.weights = ALGO == kSSSP;
     const auto body = [&](const RelaxTask &t) {
         return [&st, &t, hub_rep](const Edge<false> (&ed)[kSteps], unsigned long long) {
             relax_edges<ALGO>(st, t, ed, hub_rep);
         };
     };
     for (unsigned long long r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < na + nb; r += nwarps) {
-        if (r < na) walk_run<kSteps, false>(la, va, ta, r, sh, 0ull, ea, la_ct, body(ta));
-        else walk_run<kSteps, false>(la, vb, tb, r - na, sh, 0ull, eb, lb_ct, body(tb));
+        if (r < na) walk_run<kSteps, false, ALGO == kSSSP>(la, va, ta, r, sh, 0ull, ea, la_ct, body(ta));
+        else walk_run<kSteps, false, ALGO == kSSSP>(la, vb, tb, r - na, sh, 0ull, eb, lb_ct, body(tb));
     }
     flush_link(la_ct, ta.link_ctr);
     flush_link(lb_ct, tb.link_ctr);
 }
 
+template <bool WEIGHTS>
 __global__ void __launch_bounds__(kRelaxBlock) k_gather(ListArrays la, const Summary *sum,
                                                         RelaxTask t, unsigned int *out_dst,
                                                         unsigned int *out_w, const LoopCtl *loop) {
@@ -129,16 +201,16 @@ __global__ void __launch_bounds__(kRelaxBlock) k_gather(ListArrays la, const Sum
     unsigned long long kb, ke;
     const RouteView rv = task_view(t, sum, kb, ke);
     LinkCount lc;
-    lc.weights = out_w != nullptr;
-    walk_task<kSteps, false>(la, rv, t, kb, ke, lc, [&](const Edge<false> (&ed)[kSteps], unsigned long long k) {
+    walk_task<kSteps, false, WEIGHTS>(la, rv, t, kb, ke, lc,
+                                      [&](const Edge<false> (&ed)[kSteps], unsigned long long k) {
         unsigned int dv[kSteps], wv[kSteps] = {};
-        load_entries(t.src.dst, t.src.dst_bits, t.src.dst_off, ed, dv);
-        if (out_w) load_entries(t.src.w, t.src.w_bits, t.src.w_off, ed, wv);
+        load_entries<false>(t.src.dst, t.src.dst_bits, ed, dv);
+        if (WEIGHTS) load_entries<true>(t.src.w, t.src.w_bits, ed, wv);
 #pragma unroll
         for (int q = 0; q < kSteps; ++q) {
             if (ed[q].ok) {
                 out_dst[k + 32 * q - kb] = dv[q];
-                if (out_w) out_w[k + 32 * q - kb] = wv[q];
+                if (WEIGHTS) out_w[k + 32 * q - kb] = wv[q];
             }
         }
     });
@@ -272,8 +344,45 @@ cudaError_t launch_second_pass(const AlgoState &st, const unsigned long long *of
     return launch_relax(st, la, sum, sp_push_task(r), r.E1 > r.E0 ? (int)run_blocks(0, r.E1 - r.E0, 8 * device_sms()) : 1, s);
 }
 
+// Hub ids that a PageRank relax of at most `edges` edges sums in shared memory,
+// a multiple of 4; 0: the plain relax with replicas.  A block's sums cost its
+// share of the flush (a vector reduction per 4 ids), so the number follows the
+// edges an SM gets.  PageRank, every partition resident, plain / 4,096 / 16,384:
+// R-MAT 18 (4.2 M edges) 8.0 / 6.4 / 6.9 ms, R-MAT 19 13.1 / 11.0 / 9.3, R-MAT 21
+// 37.0 / - / 27.4; R-MAT 12 (65 K edges) 5.4 / 3.2.
+static unsigned int rank_ids(const AlgoState &st, unsigned long long edges) {
+    if ((st.algo != kPR && st.algo != kPPR) || !st.hub_rep || st.V < 4 * kRankHot || edges < kRankNarrow) return 0;
+    if (edges >= kRankWide && st.V >= 16384) return 16384;
+    return st.V >= 4096 ? 4096u : (unsigned int)st.V & ~3u;
+}
+
+// 16,384 ids: one block of 1,024 threads per SM (the cache, and its second
+// pass).  Fewer: two blocks of 512, so that another stream's task can have half
+// of an SM while this one starts or ends (PPR on R-MAT 24, F tasks of 4 M edges:
+// 209 ms, with blocks of 1,024 210 ms, of 256 217 ms).
+template <bool TB>
+static cudaError_t launch_rank(unsigned int ns, const AlgoState &st, const ListArrays &la, const Summary *sum,
+                               const RelaxTask &ta, const RelaxTask &tb, cudaStream_t s) {
+    if (ns == 16384) {
+        // above the 48 KiB that need no opt-in; the attribute is per device and
+        // setting it again is free
+        cudaError_t e = cudaFuncSetAttribute(k_relax_rank<1024, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)rank_smem(16384));
+        if (e != cudaSuccess) return e;
+        k_relax_rank<1024, TB><<<device_sms(), 1024, rank_smem(ns), s>>>(st, la, sum, ta, tb, ns);
+    } else {
+        k_relax_rank<512, TB><<<2 * device_sms(), 512, rank_smem(ns), s>>>(st, la, sum, ta, tb, ns);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_relax(const AlgoState &st, const ListArrays &la, const Summary *sum,
                          const RelaxTask &t, int grid_cap, cudaStream_t s) {
+    // edges that the task can have at most: its host bounds, or its source's
+    const unsigned long long most =
+        !t.device_sized && !t.dev_edge ? (t.k_end > t.k_begin ? t.k_end - t.k_begin : 0ull)
+        : t.route == kRouteZ && !t.sp_cursor ? 0ull : t.src.e_hi - t.src.e_lo;
+    if (const unsigned int ns = rank_ids(st, most)) return launch_rank<false>(ns, st, la, sum, t, t, s);
     unsigned int grid = (unsigned int)grid_cap;
     if (!t.device_sized && !t.dev_edge) {
         if (t.k_begin >= t.k_end) return t.sp_reset ? cudaMemsetAsync(t.sp_reset, 0, 8, s) : cudaSuccess;
@@ -290,6 +399,7 @@ cudaError_t launch_relax(const AlgoState &st, const ListArrays &la, const Summar
 
 cudaError_t launch_relax_pair(const AlgoState &st, const ListArrays &la, const Summary *sum,
                               const RelaxTask &ta, const RelaxTask &tb, int grid, cudaStream_t s) {
+    if (const unsigned int ns = rank_ids(st, ta.src.e_hi - ta.src.e_lo)) return launch_rank<true>(ns, st, la, sum, ta, tb, s);
     switch (st.algo) {
         case kBFS: k_relax_pair<kBFS><<<grid, kRelaxBlock, 0, s>>>(st, la, sum, ta, tb); break;
         case kSSSP: k_relax_pair<kSSSP><<<grid, kRelaxBlock, 0, s>>>(st, la, sum, ta, tb); break;
@@ -307,7 +417,8 @@ cudaError_t launch_gather(const ListArrays &la, const Summary *sum, const RelaxT
         if (t.k_begin >= t.k_end) return cudaSuccess;
         grid = run_blocks(t.k_begin, t.k_end, grid);
     }
-    k_gather<<<grid, kRelaxBlock, 0, s>>>(la, sum, t, out_dst, out_w, loop);
+    if (out_w) k_gather<true><<<grid, kRelaxBlock, 0, s>>>(la, sum, t, out_dst, out_w, loop);
+    else k_gather<false><<<grid, kRelaxBlock, 0, s>>>(la, sum, t, out_dst, out_w, loop);
     return cudaGetLastError();
 }
 

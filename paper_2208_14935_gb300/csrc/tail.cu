@@ -61,6 +61,12 @@ struct TailShared {
 };
 enum : unsigned int { kTailOver = 1u, kTailStop = 2u };
 
+struct TailEdge {
+    bool ok, adj;
+    long long e;                        // CSR index
+    unsigned int pay;
+};
+
 struct TailTotals {
     unsigned long long parts[kRoutes], entries[kRoutes], edges[kRoutes], lines[kRoutes];
 };
@@ -69,7 +75,7 @@ struct TailTotals {
 // the host's, both indexed from edge 0): load_entries with a pointer per edge.
 template <int S>
 __device__ __forceinline__ void tail_entries(const unsigned int *const (&p)[S], unsigned int bits,
-                                             const Edge<false> (&ed)[S], unsigned int (&out)[S]) {
+                                             const TailEdge (&ed)[S], unsigned int (&out)[S]) {
     const unsigned int mask = 0xffffffffu >> (32 - bits);
     unsigned int lo[S], hi[S], sh[S];
 #pragma unroll
@@ -139,7 +145,6 @@ __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThrea
     cl.sync();
 
     LinkCount lz, lc;                               // zero-copy and compaction routes
-    lz.weights = lc.weights = ALGO == kSSSP;
     int cur = 0, why = kTailAgain;
     bool took = false, elig = false;
     unsigned int v = 0;
@@ -236,7 +241,7 @@ __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThrea
         const unsigned int cached =
             __ballot_sync(0xffffffffu, lane < nl && mypart < a.cp.n_cached && a.cp.force_route != kRouteZ);
         // a step group's edges, targets, weights and values seen
-        Edge<false> ed[kTailSteps];
+        TailEdge ed[kTailSteps];
         int own[kTailSteps];
         unsigned int dv[kTailSteps], wv[kTailSteps] = {}, seen[kTailSteps];
         const auto load = [&](unsigned int b0) {
