@@ -835,6 +835,25 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     uint64_t n_slots = stage_cap / std::max<uint64_t>(1, bytes(slot_edges));
     n_slots = std::max<uint64_t>(1, std::min<uint64_t>({n_slots, (uint64_t)(c->streams + c->prefetch_slots),
                                                         (uint64_t)kMaxSlots}));
+    // With one or two slots a task's copy waits for the relax of the one before
+    // it, so the same bytes become three smaller slots when they still hold a
+    // partition each.  CC on R-MAT 20 at a 25 % budget, one slot against three:
+    // 1.91 / 1.43 ms; 64-source BFS 3.03 / 2.75; PageRank 40 / 29 ms.  PageRank
+    // and PPR keep larger tasks when the slots are small: a copy of a few MB is
+    // short beside the relax and second pass, which then only become more and
+    // smaller launches (32-seed PPR on R-MAT 18, 2.4 MB: 48 / 53 ms).
+    const bool rank = c->last_run_algo == kPR || c->last_run_algo == kPPR;
+    const uint64_t region = n_slots * bytes(slot_edges);
+    if (n_slots < 3 && (!rank || region >= (8u << 20))) {
+        const unsigned int ebits = c->dst_bits + (n_arrays == 2 ? c->w_bits : 0);
+        for (uint64_t want = 3; want > n_slots; --want) {
+            const uint64_t each = region / want, edges = each > slack ? (each - slack) * 8 / ebits : 0;
+            if (edges < min_slot || edges < pe || bytes(edges) > each) continue;
+            slot_edges = edges;
+            n_slots = want;
+            break;
+        }
+    }
     const uint64_t staged = n_slots * bytes(slot_edges);
     uint64_t rem = B > staged ? B - staged : 0;
     uint64_t compact_edges = std::max<uint64_t>(compact_min, (uint64_t)(B * c->compact_frac) / eb);
@@ -2956,6 +2975,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     if (s != HYTG_OK) return s;
     c->batch_mode = mode;
     c->batch_K = n_slots;
+    c->last_run_algo = algo;
     c->have_result = false;
     c->stats = hytg_stats{};
     c->iters.clear();
