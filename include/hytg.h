@@ -306,10 +306,11 @@ hytg_status hytg_run(hytg_ctx *ctx, hytg_algo algo, const uint32_t *sources, uin
 hytg_status hytg_fetch_result(hytg_ctx *ctx, void *out, uint64_t out_bytes);
 
 /* hytg_run, then hytg_fetch_result into `out` if it succeeded, in one call:
- * host threads of the context fault in the pages of `out` (their contents
- * stay) while the run is on the device, so that the copy does not take the
+ * host threads of the context fault in the pages of `out`, with a store to
+ * each, while the run is on the device, so that the copy does not take the
  * page faults of a fresh allocation one at a time.  `out` must stay valid
- * until the call returns; arguments and errors are those of the two calls. */
+ * until the call returns; after an error its first 4*V*n_sources bytes are
+ * undefined.  Arguments and errors are those of the two calls. */
 hytg_status hytg_run_fetch(hytg_ctx *ctx, hytg_algo algo, const uint32_t *sources, uint32_t n_sources,
                            void *out, uint64_t out_bytes);
 

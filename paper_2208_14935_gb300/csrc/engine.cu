@@ -124,14 +124,15 @@ private:
 // fills it is on the device.  A caller's fresh allocation has no pages yet, and
 // a device-to-host copy into it spends most of its time on page faults taken
 // one at a time (256 MiB: 9.6 ms, against 1.4 ms into present pages; 64 MiB: 2.6
-// and 0.37 ms).  The pages are populated for writing by the kernel call for
-// that, which leaves their contents alone; reading a byte and writing it back
-// would map the zero page first and then replace it, and that replacement,
-// which the device's view of the page tables must follow, made a 64-source BFS
-// take 106 ms instead of 15.  Whole calls, faults in the copy -> after the run
-// from eight threads -> beside the run: 64-source BFS on R-MAT 20 14.8 ->
-// 11.3 -> 8.3 ms, BFS on R-MAT 24 7.9 -> 6.6 -> 5.1 ms.  start() returns at
-// once; finish() helps, and returns when every page is present.
+// and 0.37 ms).  A plain store per page it is: reading the byte first would map
+// the zero page and then replace it, and that replacement, which the device's
+// view of the page tables must follow, made a 64-source BFS take 106 ms instead
+// of 15; populating ranges by madvise keeps the contents but takes twice as
+// long (256 MiB from eight threads: 5.2 ms, stores 2.4).  So the buffer's
+// contents are lost from the start.  Whole calls, faults in the copy -> stores
+// beside the run: 64-source BFS on R-MAT 20 14.8 -> 6.1 ms, BFS on R-MAT 24
+// 7.9 -> 5.1 ms.  start() returns at once; finish() helps, and returns when every
+// page is present.
 class PageToucher {
 public:
     explicit PageToucher(unsigned n) {
@@ -162,15 +163,16 @@ public:
 
 private:
     static constexpr size_t kPiece = size_t(1) << 21;
-    static constexpr int kPopulateWrite = 23;        // MADV_POPULATE_WRITE (Linux 5.14)
     void work() {
         static const size_t page = (size_t)std::max<long>(4096, sysconf(_SC_PAGESIZE));
         for (;;) {
             const size_t lo = next_.fetch_add(kPiece);
             if (lo >= bytes_) return;
             const size_t hi = std::min(bytes_, lo + kPiece);
-            const uintptr_t a = ((uintptr_t)p_ + lo) & ~(uintptr_t)(page - 1);
-            madvise((void *)a, (uintptr_t)p_ + hi - a, kPopulateWrite);
+            // the piece's first byte, then every page that starts inside it
+            volatile char *p = p_;
+            p[lo] = 0;
+            for (size_t q = lo + (page - (((uintptr_t)p + lo) & (page - 1))); q < hi; q += page) p[q] = 0;
         }
     }
     void loop() {
