@@ -62,7 +62,7 @@ def parse():
     ap.add_argument("--no-batched", action="store_true", help="skip the batched-vs-plain runs")
     ap.add_argument("--timeline-out", default="", metavar="PATH",
                     help="save each algorithm's launch timeline of the last timed step (numpy .npz); "
-                         "with --param device_loop=0 its k_second_pass/k_relax entries follow the "
+                         "with --param device_loop=0 its second-pass and relax entries follow the "
                          "process's launch order, so a profiler's launch index maps to an edge count")
     ap.add_argument("--mesh-only", type=int, default=0, metavar="SIDE",
                     help="only the high-diameter workload: SIDE x SIDE 4-neighbour mesh with 0.1 %% "
@@ -594,17 +594,18 @@ def main():
         rf_n, rf_ms = sum(t["rf_n"] for t in tls), sum(t["rf_ms"] for t in tls)
         rf_e = sum(t["rf_edges"] for t in tls)
         rf_v = sum(st["route_vertices"][2] for st in prs)
+        eb = max(1, (g.V - 1).bit_length()) / 8    # bytes of a packed target
         kern = {}
         if sp_n:
-            # per relaxed edge 4 B edge + 8 B value read-modify-write; per
+            # per relaxed edge its packed target + 8 B value read-modify-write; per
             # scanned vertex 16 B offsets, 4 B delta read, 8 B delta and rank updates
-            kern["k_second_pass<PageRank>"] = (sp_n, sp_ms, sp_e, sp_e * 12 + sp_v * 28,
-                                               "per edge 4 + 8 (value RMW), per scanned vertex 28",
+            kern["k_second_pass<PageRank>"] = (sp_n, sp_ms, sp_e, sp_e * (eb + 8) + sp_v * 28,
+                                               f"per edge {eb} + 8 (value RMW), per scanned vertex 28",
                                                sp_v)
         if rf_n:
-            # per edge 4 B edge + 8 B RMW, per list entry 20 B
-            kern["k_relax<PageRank> F route"] = (rf_n, rf_ms, rf_e, rf_e * 12 + rf_v * 20,
-                                                 "per edge 4 + 8 (value RMW), per active vertex 20",
+            # per edge its packed target + 8 B RMW, per list entry 20 B
+            kern["k_relax<PageRank> F route"] = (rf_n, rf_ms, rf_e, rf_e * (eb + 8) + rf_v * 20,
+                                                 f"per edge {eb} + 8 (value RMW), per active vertex 20",
                                                  rf_v)
         if kern:
             dom = max(kern, key=lambda k: kern[k][1])

@@ -403,8 +403,9 @@ hytg_status hytg_get_iterations(hytg_ctx *ctx, hytg_iter_record *out, uint32_t c
 /* One timed launch or copy of the last hytg_run ("timing" parameter 1), in
  * issue order.  Host-issued work only: iterations inside the device-loop
  * graph are not split into launches.  The second-pass entries, in order, are
- * the process's k_second_pass launches of that run, so a profiler's launch
- * index can be matched to its edge count when the device loop is off. */
+ * that run's second passes (a take and a relax of its list each), so a
+ * profiler's launch index can be matched to an edge count when the device
+ * loop is off. */
 typedef struct hytg_timed_launch {
     uint32_t kind;                    /* HYTG_K_* (HYTG_K_SECOND_PASS for a second pass) */
     uint32_t stream;                  /* 0 main stream, 1 compaction stream, 2 + i F stream i,

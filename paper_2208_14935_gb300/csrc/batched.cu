@@ -47,6 +47,7 @@ __global__ void k_b_init(BatchState b, unsigned long long V, unsigned long long 
     const unsigned long long t0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     if (b.mode == kBatchPPR) {
         for (unsigned long long v = t0; v < V; v += stride) b.fr32[v] = 0;
+        for (unsigned long long i = t0; i < kBatchHubCopies * b.n_hub * kMaxPprSeeds; i += stride) b.hub[i] = 0.0f;
     } else {
         for (unsigned long long v = t0; v < V; v += stride) {
             b.fr[v] = 0;
@@ -109,6 +110,28 @@ __global__ void k_b_commit(BatchState b, unsigned long long V, unsigned long lon
             if (lane == 0) atomicOr(b.alive, orv);
         }
     }
+}
+
+// PPR: the hub copies' sums enter the residuals (ppr_edges).  A thread per hub
+// id and seed; pushes and other folds may run meanwhile, so a copy is swapped
+// out.  The sixteen loads are in flight together, and copies without pushes
+// are left alone.
+__global__ void k_b_hub_fold(BatchState b) {
+    const unsigned int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned int v = i / kMaxPprSeeds, s = i % kMaxPprSeeds;
+    if (v >= b.n_hub || b.delta[s / kFrameSources] == nullptr) return;
+    float x[kBatchHubCopies];
+#pragma unroll
+    for (unsigned int r = 0; r < kBatchHubCopies; ++r) x[r] = __ldcg(b_hub(b, r, v, s));
+    double sum = 0.0;
+#pragma unroll
+    for (unsigned int r = 0; r < kBatchHubCopies; ++r)
+        if (x[r] != 0.0f) sum += (double)atomicExch(b_hub(b, r, v, s), 0.0f);
+    if (sum != 0.0) atomicAdd(bdelta(b, v, s), (float)sum);
+}
+cudaError_t hub_fold(const BatchState &b, cudaStream_t s) {
+    if (b.n_hub) k_b_hub_fold<<<(b.n_hub * kMaxPprSeeds + 255) / 256, 256, 0, s>>>(b);
+    return cudaGetLastError();
 }
 
 // PPR: for every vertex marked in the bitmap, take the residual of each seed
@@ -298,14 +321,22 @@ __device__ __forceinline__ void mssssp_edges(const BatchState &b, unsigned int v
 // 15 % of the edges of a 2^18-vertex graph end in the first 32 vertices, one
 // word, and as many atomics on one address took most of the relax's time.
 // Both together: 590 K edges with 32 seeds each, 260 -> 70 us (70 G vector
-// reductions/s); replica frames for the hub ids, as single-source PageRank has,
-// gained nothing after this and hid the hubs' residuals from the second passes
-// (183 iterations instead of 103 on R-MAT 18).
+// reductions/s).
+//
+// Pushes to the lowest ids go to one of sixteen copies of their rows, folded
+// before every take that looks at them.  The copies are for the rounding: a hub
+// that 10^5 equal messages reach in one iteration gathers a bias of 4e-5 in
+// one 32-bit sum (Chung-Lu 2.1, 4 M edges, resident: result off by 1.1e-5 in
+// the 2-norm), and sixteen sums of a sixteenth are each that much closer
+// (9.7e-7).  The same graph's run went from 69 to 40 ms, since one address no
+// longer takes 3 % of all pushes; R-MAT 18, whose targets are flatter, pays 3 %
+// for the test and the folds.
 // (The plain load may miss a bit set meanwhile, never see one too many: bits
 // are only cleared between relaxes, by earlier kernels of the main stream.)
 __device__ __forceinline__ void ppr_edges(const BatchState &b, unsigned int w, unsigned int u, unsigned int m,
                                           unsigned int *bm) {
     const int lane = threadIdx.x & 31, part = lane & 7, sub = lane >> 3;
+    const unsigned int copy = sm_id() % kBatchHubCopies;
     if (m && !((bm[w >> 5] >> (w & 31)) & 1u)) atomicOr(&bm[w >> 5], 1u << (w & 31));
     constexpr int kTurns = 4;                       // 16 edges' messages in flight
 #pragma unroll
@@ -321,7 +352,8 @@ __device__ __forceinline__ void ppr_edges(const BatchState &b, unsigned int w, u
             if ((me >> (4 * part)) & 0xFu) {
                 const unsigned int g = part >> 1, h = 4 * (part & 1);
                 x[i] = __ldcg((const float4 *)(b.msg[g] + (unsigned long long)ue * kFrameSources + h));
-                to[i] = b.delta[g] + (unsigned long long)we * kFrameSources + h;
+                to[i] = we < b.n_hub ? b_hub(b, copy, we, 4 * part)
+                                     : b.delta[g] + (unsigned long long)we * kFrameSources + h;
             }
         }
 #pragma unroll
@@ -494,6 +526,8 @@ cudaError_t launch_b_commit(const BatchState &b, unsigned long long V, unsigned 
 cudaError_t launch_b_take(const BatchState &b, const unsigned long long *off,
                           unsigned long long n_words_alloc, unsigned int K, float damping, float eps,
                           unsigned int *bm, cudaStream_t s) {
+    cudaError_t e = hub_fold(b, s);
+    if (e != cudaSuccess) return e;
     k_b_take<<<grid_for(n_words_alloc * 32, 256), 256, 0, s>>>(b, off, n_words_alloc, K, damping, eps, bm);
     return cudaGetLastError();
 }
@@ -520,6 +554,8 @@ cudaError_t launch_second_pass_batched(const BatchState &b, const unsigned long 
     if (r.vhi <= r.vlo) return cudaSuccess;
     if ((r.vlo & 31) || b.mode != kBatchPPR || r.vhi - r.vlo > kSpEntries || r.E1 - r.E0 > kSpEdgesMax)
         return cudaErrorInvalidValue;
+    cudaError_t e = r.vlo < b.n_hub ? hub_fold(b, s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
     k_bsp_take<<<sp_take_blocks(r.vhi - r.vlo, kRelaxBlock), kRelaxBlock, 0, s>>>(b, off, r, la, K, damping, eps);
     return launch_relax_batched(b, la, sum, sp_push_task(r),
                                 r.E1 > r.E0 ? (int)run_blocks(0, r.E1 - r.E0, 8 * device_sms()) : 1, bm, nullptr, s);
@@ -547,7 +583,8 @@ cudaError_t launch_serve_extract(const BatchState &b, unsigned long long V, unsi
 cudaError_t launch_b_finalize(const BatchState &b, unsigned long long V, unsigned int K,
                               const unsigned int *perm, void *out, double *sums, cudaStream_t s) {
     if (b.mode == kBatchPPR) {
-        cudaError_t e = cudaMemsetAsync(sums, 0, 64 * sizeof(double), s);
+        cudaError_t e = hub_fold(b, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, 64 * sizeof(double), s);
         if (e != cudaSuccess) return e;
         k_b_pr_sums<<<grid_for(V * 32, 256), 256, 0, s>>>(b, V, K, sums);
         k_b_pr_out<<<grid_for(V * K, 256), 256, 0, s>>>(b, V, K, perm, sums, (float *)out);

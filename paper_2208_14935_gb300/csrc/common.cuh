@@ -224,6 +224,8 @@ struct BatchState {
     unsigned int *val[kMaxFrames];        // BFS level / SSSP distance frames (nullptr: none)
     float *delta[kMaxPprFrames], *rank[kMaxPprFrames], *msg[kMaxPprFrames];   // PPR frames
     unsigned int *fr32;                   // PPR seeds taken at v this iteration
+    float *hub;                           // PPR pushes to ids [0, n_hub): kBatchHubCopies copies of
+    unsigned int n_hub;                   // n_hub rows of kMaxPprSeeds floats (b_hub)
     unsigned long long *alive;            // OR of every vertex's frontier mask (serving)
     const LoopCtl *loop;                  // device loop: level from loop->it; relax gated by loop->work
     unsigned int sparse_below;            // SSSP/PPR relax: a warp whose 32 edges carry fewer than
@@ -243,6 +245,11 @@ __device__ __forceinline__ float *bmsg(const BatchState &b, unsigned long long v
     return b.msg[s >> 3] + v * kFrameSources + (s & 7);
 }
 constexpr unsigned int kHubReplicas = 256;
+// Batched PPR's hub copies, in the memory of the single-source replicas.
+constexpr unsigned int kBatchHubIds = 64, kBatchHubCopies = 16, kMaxPprSeeds = kMaxPprFrames * kFrameSources;
+__device__ __forceinline__ float *b_hub(const BatchState &b, unsigned int copy, unsigned int v, unsigned int s) {
+    return b.hub + ((size_t)copy * b.n_hub + v) * kMaxPprSeeds + s;
+}
 
 // log2 of a power of two, else -1.
 inline int log2_exact(unsigned long long m) {

@@ -1275,6 +1275,11 @@ hytg_status ensure_batch(hytg_ctx *c, int mode, uint32_t out_rows) {
     }
     c->bs.mode = mode;
     c->bs.alive = c->d_alive;
+    // hub copies of batched PPR: in the single-source replicas, which no run of
+    // the other kind uses meanwhile, as many ids as fit there
+    static_assert(kBatchHubCopies * kMaxPprSeeds == 2 * kHubReplicas, "a batched id takes the room of two");
+    c->bs.hub = mode == kBatchPPR ? c->d_hub_rep : nullptr;
+    c->bs.n_hub = c->bs.hub ? std::min(kBatchHubIds, c->n_hub_rep / 2) : 0;
     c->bs.sparse_below = c->batch_sparse_below >= 0 ? (unsigned int)c->batch_sparse_below : 16u;
     for (auto &p : c->bs.val) p = nullptr;
     for (uint32_t g = 0; g < kMaxPprFrames; ++g) c->bs.delta[g] = c->bs.rank[g] = c->bs.msg[g] = nullptr;
