@@ -135,8 +135,12 @@ private:
 // page is present.
 class PageToucher {
 public:
+    // As many threads as can be had: finish() does what they leave.
     explicit PageToucher(unsigned n) {
-        for (unsigned i = 0; i < n; ++i) th_.emplace_back([this] { loop(); });
+        try {
+            for (unsigned i = 0; i < n; ++i) th_.emplace_back([this] { loop(); });
+        } catch (...) {
+        }
     }
     ~PageToucher() {
         { std::lock_guard<std::mutex> l(mu_); stop_ = true; }
@@ -1448,9 +1452,9 @@ bool loop_applies(const hytg_ctx *c) {
 }
 
 // F and C iterations can stay in the device loop: batched runs at "device_loop"
-// 1 (PPR: of graphs up to kLoopFcEdges edges), every run at 2; not with host compaction, forced random routes, more
-// partitions than 1024 IF nodes, or a staging slot without room for one
-// partition.
+// 1 (PPR: of graphs up to kLoopFcEdges edges), every run at 2; not with host
+// compaction, forced random routes, more partitions than 1024 IF nodes, or a
+// staging slot without room for one partition.
 //
 // A partition's IF node costs about 1 us per iteration closed and 20 to 40 us
 // open, copies one partition at a time and shares one chain of launches per
@@ -2274,9 +2278,16 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
 }
 
 // Start faulting in a result buffer's pages; false if it is too small to be
-// worth waking the threads for or they cannot be made.
+// worth waking the threads for, is device memory (the copy refuses that), or
+// the threads' state cannot be made.
 bool touch_start(hytg_ctx *c, void *out, uint64_t bytes) {
     if (bytes < (4u << 20)) return false;
+    cudaPointerAttributes at{};
+    if (cudaSetDevice(c->device) != cudaSuccess || cudaPointerGetAttributes(&at, out) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (at.type == cudaMemoryTypeDevice) return false;
     if (!c->toucher) {
         try {
             c->toucher = new PageToucher(std::max(1u, std::min(7u, std::thread::hardware_concurrency())));
