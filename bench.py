@@ -611,15 +611,12 @@ def main():
             dom = max(kern, key=lambda k: kern[k][1])
             n, ms, e_, alg, model, vv = kern[dom]
             achieved = alg / (ms * 1e-3) / 1e9
-            traffic, note = None, "no ncu DRAM capture of the current kernel"
-            if dom.startswith("k_second_pass"):
-                # DRAM bytes from one cold-cache ncu capture of each of its two
-                # launches on R-MAT 22: the push read 29.8 MB for 4,183,639
-                # edges, the take 0.43 MB for 22,240 vertices; scaled to this
-                # run's mean launch by its edges and vertices
-                traffic = (29.778176e6 / 4183639) * (e_ / n) + (430592.0 / 22240) * (vv / n)
-                note = ("scaled from ncu captures on R-MAT 22 (push 7.12 B/edge, take 19.4 B/vertex, "
-                        "cold cache) by this run's edges and vertices per launch")
+            # DRAM bytes of both kernels' relax from one ncu capture of its dense
+            # launch on R-MAT 22: 245.7 MB for 67,108,864 edges; scaled to this
+            # run's mean launch by its edges
+            traffic = 245730048 / 67108864 * (e_ / n)
+            note = ("scaled from an ncu capture of k_relax_rank on R-MAT 22 (3.66 B/edge) by this run's "
+                    "edges per launch" + (", without the take" if dom.startswith("k_second_pass") else ""))
             roofline = {"kernel": dom, "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                         "frac": achieved / hbm, "traffic": traffic, "traffic_note": note,
                         "bytes_model": model, "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_src})",
