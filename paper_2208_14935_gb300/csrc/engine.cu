@@ -263,7 +263,6 @@ struct hytg_ctx {
 
     // batched runs (several sources in one run, sharing every transfer)
     BatchState bs{};
-    bool bs_alloc_mask = false, bs_alloc_ppr = false;
     unsigned int *own_val[kMaxFrames] = {};              // hytg_run's BFS/SSSP frames (V * 32 B each)
     float *own_ppr[kMaxPprFrames] = {};                  // hytg_run's PPR frames (V * 96 B each)
     int batch_mode = kBatchNone;
@@ -453,6 +452,28 @@ void dfree(T *&p) {
     p = nullptr;
 }
 
+// `bytes` of device memory for p, unless it has some already.  Arrays made on
+// first use go through here one by one, so that after a call that ran out of
+// memory half way the next one makes what is missing; the failure is this
+// call's and is not left behind as CUDA's last error for the next launch.
+// HYTG_INJECT_DEVMEM_FAIL=<name> fails the array of that name, for tests.
+template <typename T>
+hytg_status ensure_dev(hytg_ctx *c, T *&p, uint64_t bytes, const char *name) {
+    if (p) return HYTG_OK;
+    const char *inject = getenv("HYTG_INJECT_DEVMEM_FAIL");
+    const cudaError_t e = inject && !std::strcmp(inject, name) ? cudaErrorMemoryAllocation
+                                                               : cudaMalloc((void **)&p, bytes);
+    if (e == cudaSuccess) return HYTG_OK;
+    p = nullptr;
+    (void)cudaGetLastError();
+    return fail(c, HYTG_ERR_CUDA, std::string("device allocation of ") + name + ": " + cudaGetErrorString(e));
+}
+#define ENSURE(p, bytes)                                                 \
+    do {                                                                 \
+        const hytg_status _s = ensure_dev(c, p, (bytes), &(#p)[3]);      \
+        if (_s != HYTG_OK) return _s;                                    \
+    } while (0)
+
 void free_loop_graph(hytg_ctx *c) {
     if (c->loop_exec) cudaGraphExecDestroy(c->loop_exec);
     if (c->loop_graph) cudaGraphDestroy(c->loop_graph);
@@ -590,7 +611,6 @@ void free_graph(hytg_ctx *c) {
     for (auto &f : c->own_val) dfree(f);
     for (auto &f : c->own_ppr) dfree(f);
     c->bs = BatchState{};
-    c->bs_alloc_mask = c->bs_alloc_ppr = false;
     c->batch_mode = kBatchNone;
     c->permuted = false;
     c->n_hubs = 0;
@@ -1152,27 +1172,37 @@ bool second_pass_on(const hytg_ctx *c, int algo) {
     return c->two_pass == 2 || algo == kPR || algo == kPPR;
 }
 
+// The tile index of the second passes: a range's slice starts at its first edge's
+// tile plus its first partition's number (second_pass_any).
+uint64_t sp_tile_count(const hytg_ctx *c) { return c->E / kTile + (c->part_vb.size() - 1) + 2; }
+
 // Arrays of the second passes, allocated by the first run that has them and
 // kept with the graph (vertex-side data, outside the budget).
 hytg_status ensure_second_pass(hytg_ctx *c, int algo) {
     if (!second_pass_on(c, algo)) return HYTG_OK;
     const uint64_t N = c->part_vb.size() - 1;
-    if (!c->d_sp_ebase) {
-        CK(cudaMalloc(&c->d_sp_ebase, c->V * 8));
-        CK(cudaMalloc(&c->d_sp_soff, c->V * 8));
-        c->vertex_bytes += c->V * 16;
-    }
+    ENSURE(c->d_sp_ebase, c->V * 8);
+    ENSURE(c->d_sp_soff, c->V * 8);
+    c->sp_tiles = sp_tile_count(c);
+    ENSURE(c->d_sp_tiles, c->sp_tiles * 4);
     if (!c->d_sp_cursor) {
-        c->sp_tiles = c->E / kTile + N + 2;
-        CK(cudaMalloc(&c->d_sp_tiles, c->sp_tiles * 4));
-        CK(cudaMalloc(&c->d_sp_cursor, N * 8));
-        CK(cudaMemset(c->d_sp_cursor, 0, N * 8));
+        ENSURE(c->d_sp_cursor, N * 8);
+        const cudaError_t e = cudaMemset(c->d_sp_cursor, 0, N * 8);
+        if (e != cudaSuccess) dfree(c->d_sp_cursor);    // cleared, or not there
+        CK(e);
     }
-    if (c->batch_mode == kBatchPPR && !c->d_sp_pay64) {
-        CK(cudaMalloc(&c->d_sp_pay64, c->V * 8));
-        CK(cudaMalloc(&c->d_sp_vid, c->V * 4));
+    if (c->batch_mode == kBatchPPR) {
+        ENSURE(c->d_sp_pay64, c->V * 8);
+        ENSURE(c->d_sp_vid, c->V * 4);
     }
     return HYTG_OK;
+}
+
+// Device bytes of the second passes' arrays that have been made.
+uint64_t second_pass_bytes(const hytg_ctx *c) {
+    const uint64_t N = c->part_vb.size() - 1;
+    return (c->d_sp_ebase ? c->V * 8 : 0) + (c->d_sp_soff ? c->V * 8 : 0) + (c->d_sp_pay64 ? c->V * 8 : 0) +
+           (c->d_sp_vid ? c->V * 4 : 0) + (c->d_sp_tiles ? c->sp_tiles * 4 : 0) + (c->d_sp_cursor ? N * 8 : 0);
 }
 
 // Partitions [i, j) of one second-pass list: as many as the packed cursor
@@ -1256,26 +1286,20 @@ cudaError_t relax_any(hytg_ctx *c, const AlgoState &st, const ListArrays &la, co
 // frame pointer is cleared; attach_own_frames or the serving calls set them.
 hytg_status ensure_batch(hytg_ctx *c, int mode, uint32_t out_rows) {
     const uint64_t V = c->V;
-    if (!c->d_pay64) {
-        CK(cudaMalloc(&c->d_pay64, V * 8));
-        CK(cudaMalloc(&c->d_vid, V * 4));
-    }
+    ENSURE(c->d_pay64, V * 8);
+    ENSURE(c->d_vid, V * 4);
     if (c->bout_rows < out_rows) {
         dfree(c->d_bout);
         c->bout_rows = 0;
-        CK(cudaMalloc(&c->d_bout, V * 4 * out_rows));
+        ENSURE(c->d_bout, V * 4 * out_rows);
         c->bout_rows = out_rows;
     }
     if (mode == kBatchPPR) {
-        if (!c->bs_alloc_ppr) {
-            CK(cudaMalloc(&c->bs.fr32, V * 4));
-            c->bs_alloc_ppr = true;
-        }
-    } else if (!c->bs_alloc_mask) {
-        CK(cudaMalloc(&c->bs.fr, V * 8));
-        CK(cudaMalloc(&c->bs.vis, V * 8));
-        CK(cudaMalloc(&c->bs.nxt, V * 8));
-        c->bs_alloc_mask = true;
+        ENSURE(c->bs.fr32, V * 4);
+    } else {
+        ENSURE(c->bs.fr, V * 8);
+        ENSURE(c->bs.vis, V * 8);
+        ENSURE(c->bs.nxt, V * 8);
     }
     c->bs.mode = mode;
     c->bs.alive = c->d_alive;
@@ -1323,7 +1347,8 @@ hytg_status attach_own_frames(hytg_ctx *c, int mode, uint32_t K) {
     const uint32_t groups = (K + kFrameSources - 1) / kFrameSources;
     for (uint32_t g = 0; g < groups; ++g) {
         void **own = mode == kBatchPPR ? (void **)&c->own_ppr[g] : (void **)&c->own_val[g];
-        if (!*own) CK(cudaMalloc(own, frame_bytes(c, mode)));
+        const hytg_status s = ensure_dev(c, *own, frame_bytes(c, mode), "frame");
+        if (s != HYTG_OK) return s;
         set_group_frame(c, g, (char *)*own);
     }
     return HYTG_OK;
@@ -3035,7 +3060,10 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     for (auto &f : c->serve_group_frame) f = -1;
     s = ensure_cache(c, n_arrays);
     if (s == HYTG_OK) s = ensure_second_pass(c, algo);
-    if (s != HYTG_OK) return s;
+    if (s != HYTG_OK) {
+        c->batch_mode = kBatchNone;                  // no session
+        return s;
+    }
     CK(cudaMemsetAsync(c->d_report, 0, offsetof(RunReport, sp), c->s_main));
     CK(launch_b_init(c->bs, c->V, c->n_words_alloc, c->d_src, 0, 0.0f, c->d_bm[0], c->s_main));
     c->serving = true;
@@ -3211,7 +3239,7 @@ hytg_status hytg_get_info(hytg_ctx *c, hytg_info *out) {
     i.budget_bytes = c->budget;
     i.budget_used_bytes = c->carve.used;
     i.compact_edges = c->carve.compact_edges;
-    i.vertex_state_bytes = c->loaded ? c->vertex_bytes : 0;
+    i.vertex_state_bytes = c->loaded ? c->vertex_bytes + second_pass_bytes(c) : 0;
     i.pinned_host_bytes = c->loaded ? 4 * (packed_words(c->E, c->dst_bits) +
                                            (c->weighted ? packed_words(c->E, c->w_bits) : 0)) : 0;
     *out = i;
