@@ -2627,6 +2627,7 @@ hytg_status hytg_set_param(hytg_ctx *c, const char *key, double v) {
         c->part_bytes = v;
         if (c->loaded) {
             CK(cudaSetDevice(c->device));
+            CK(cudaDeviceSynchronize());             // a serving step's tasks read the old arrays
             c->part_edges = std::max<uint64_t>(1, (uint64_t)(v / 4));
             make_partitions(c);
             hytg_status s = upload_partitions(c);
@@ -3041,7 +3042,8 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
             why = c->err;
             continue;
         }
-        const uint64_t base = (c->carve.end + 255) & ~uint64_t(255);
+        // behind any carve of eb, so that a step may carve again
+        const uint64_t base = (eb + kPoolSlack + 255) & ~uint64_t(255);
         if (base + (uint64_t)nf * fb > pool_bytes) continue;
         c->serve_frame_base = (char *)c->d_pool + base;
         c->serve_edge_budget = eb;
@@ -3110,7 +3112,18 @@ hytg_status hytg_serve_step(hytg_ctx *c, uint64_t *finished, uint64_t *busy) {
         const int algo = c->serve_algo;
         const int n_arrays = algo == kSSSP ? 2 : 1;
         const uint32_t it = c->serve_it;
-        hytg_status s = issue_plan(c, algo, 0xFFFFFFFFu, it, it & 1, true);
+        // a parameter set since the last step may have undone the carve
+        // ("part_bytes", "k", "streams", ...) or switched the second pass on
+        hytg_status s = HYTG_OK;
+        if (c->carve.n_arrays == 0) {
+            CK(cudaDeviceSynchronize());             // the last step's tasks read the old slots
+            CK(ahead_drop(c));
+            s = plan_carve(c, n_arrays, c->serve_edge_budget);
+            if (s == HYTG_OK) s = ensure_cache(c, n_arrays);
+        }
+        if (s == HYTG_OK) s = ensure_second_pass(c, algo);
+        if (s != HYTG_OK) return s;
+        s = issue_plan(c, algo, 0xFFFFFFFFu, it, it & 1, true);
         if (s != HYTG_OK) return s;
         CK(cudaEventSynchronize(c->ev_sum[it & 1]));
         const char *hb = (const char *)c->h_sumbuf[it & 1];
