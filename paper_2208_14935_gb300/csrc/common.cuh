@@ -156,7 +156,7 @@ struct LoopCtl {
     unsigned long long c_cap;       // compaction buffer, in edges (larger C routes go to the host)
     const unsigned char *route;     // per-partition routes of the iteration
     const unsigned long long *part_eb;
-    unsigned int n_parts, n_arrays;
+    unsigned int n_parts, dst_bits, w_bits;   // w_bits 0: the run reads no weights
     // a word of mapped host memory that the host sets to end the loop at the
     // next iteration boundary (a run past its deadline); nullptr: none
     const volatile unsigned int *cancel;
@@ -288,6 +288,16 @@ struct EdgeSrc {
     long long dst_off, w_off;
     unsigned long long e_lo, e_hi;      // edges present: [e_lo, e_hi)
 };
+
+// The words to copy for entries [e0, e0 + n) of `bits` bits: from the 16-byte
+// boundary at or below the first entry to the word of the last one.
+struct WordSpan {
+    unsigned long long w0, n;
+};
+__host__ __device__ inline WordSpan word_span(unsigned long long e0, unsigned long long n, unsigned int bits) {
+    const unsigned long long w0 = (e0 * bits / 32) & ~3ull;
+    return {w0, n ? ((e0 + n) * bits + 31) / 32 - w0 : 0};
+}
 
 struct RelaxTask {
     int route;                          // which route's list / tiles

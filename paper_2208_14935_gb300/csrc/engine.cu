@@ -495,16 +495,6 @@ unsigned int bits_for(uint64_t max_value) {
 // entry's second word) and rounded to 16 bytes.
 uint64_t packed_words(uint64_t n, unsigned int bits) { return ((n * bits + 31) / 32 + 1 + 3) & ~uint64_t(3); }
 
-// The words to copy for entries [e0, e0 + n): from the 16-byte boundary at or
-// below the first entry to the word of the last one.
-struct WordSpan {
-    uint64_t w0, n;
-};
-WordSpan word_span(uint64_t e0, uint64_t n, unsigned int bits) {
-    const uint64_t w0 = (e0 * bits / 32) & ~uint64_t(3);
-    return {w0, n ? ((e0 + n) * bits + 31) / 32 - w0 : 0};
-}
-
 inline uint32_t packed_get(const uint32_t *a, unsigned int bits, uint64_t e) {
     const uint64_t bit = e * bits;
     const unsigned int sh = (unsigned int)(bit & 31);
@@ -2244,7 +2234,8 @@ hytg_status run_device_loop(hytg_ctx *c, uint32_t &it, unsigned int &bucket, uin
         h.route = pa.route;
         h.part_eb = c->d_part_eb;
         h.n_parts = (unsigned int)(c->part_vb.size() - 1);
-        h.n_arrays = c->last_run_arrays;
+        h.dst_bits = c->dst_bits;
+        h.w_bits = c->last_run_arrays == 2 ? c->w_bits : 0;
     }
     h.cancel = c->has_deadline ? c->d_cancel : nullptr;
     if (c->loop_fc) {

@@ -397,7 +397,9 @@ __device__ void loop_decide(const Summary *sum, LoopCtl *ctl, unsigned long long
             cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->f_handles[i], f ? 1u : 0u);
             if (f) {
                 ++np;
-                nb += (ctl->part_eb[i + 1] - ctl->part_eb[i]) * 4ull * ctl->n_arrays;
+                const unsigned long long e0 = ctl->part_eb[i], n = ctl->part_eb[i + 1] - e0;
+                nb += 4 * word_span(e0, n, ctl->dst_bits).n;
+                if (ctl->w_bits) nb += 4 * word_span(e0, n, ctl->w_bits).n;
             }
         }
         if (np) {
