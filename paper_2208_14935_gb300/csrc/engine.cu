@@ -819,7 +819,10 @@ void slots_forget(hytg_ctx *c) {
     for (auto &h : c->slot_held) h = hytg_ctx::SlotHeld();
 }
 
-hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
+// For runs of `algo`, whatever ran before; the resident prefix depends on the
+// arrays that it reads alone.
+hytg_status plan_carve(hytg_ctx *c, int algo, uint64_t edge_budget = 0) {
+    const int n_arrays = algo == kSSSP ? 2 : 1;
     const uint64_t B = edge_budget ? edge_budget : c->budget;
     Carve &cv = c->carve;
     const uint64_t pe = c->part_edges;
@@ -858,7 +861,7 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
     // and PPR keep larger tasks when the slots are small: a copy of a few MB is
     // short beside the relax and second pass, which then only become more and
     // smaller launches (32-seed PPR on R-MAT 18, 2.4 MB: 48 / 53 ms).
-    const bool rank = c->last_run_algo == kPR || c->last_run_algo == kPPR;
+    const bool rank = algo == kPR || algo == kPPR;
     const uint64_t region = n_slots * bytes(slot_edges);
     if (n_slots < 3 && (!rank || region >= (8u << 20))) {
         const unsigned int ebits = c->dst_bits + (n_arrays == 2 ? c->w_bits : 0);
@@ -870,8 +873,9 @@ hytg_status plan_carve(hytg_ctx *c, int n_arrays, uint64_t edge_budget = 0) {
             break;
         }
     }
-    const uint64_t staged = n_slots * bytes(slot_edges);
-    uint64_t rem = B > staged ? B - staged : 0;
+    // what is left is the same however the region is split, so that runs of two
+    // algorithms in turn keep one cache
+    uint64_t rem = B > region ? B - region : 0;
     uint64_t compact_edges = std::max<uint64_t>(compact_min, (uint64_t)(B * c->compact_frac) / eb);
     compact_edges = std::min<uint64_t>(compact_edges, rem / eb);
     compact_edges = compact_edges / kCompactUnit * kCompactUnit;
@@ -2593,7 +2597,7 @@ hytg_status hytg_set_device_budget(hytg_ctx *c, uint64_t bytes) {
     CK(cudaMalloc(&c->d_pool, bytes + kPoolSlack));
     c->budget = bytes;
     if (c->loaded) {
-        hytg_status s = plan_carve(c, 1);
+        hytg_status s = plan_carve(c, kBFS);
         if (s == HYTG_ERR_BUDGET) {
             // keep the pool; the error is reported again by hytg_run
             return s;
@@ -2758,7 +2762,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         c->last_run_arrays = n_arrays;
         c->last_run_algo = algo;
         CK(cudaEventRecord(c->ev_run[0], c->s_main));
-        hytg_status s = plan_carve(c, n_arrays);
+        hytg_status s = plan_carve(c, algo);
         if (s != HYTG_OK) return s;
         s = ensure_cache(c, n_arrays);
         if (s == HYTG_OK) s = ensure_second_pass(c, algo);
@@ -3029,7 +3033,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     for (; nf >= 1; --nf) {
         if ((uint64_t)nf * fb + kPoolSlack >= c->budget) continue;
         const uint64_t eb = c->budget - (uint64_t)nf * fb - kPoolSlack;
-        if (plan_carve(c, n_arrays, eb) != HYTG_OK) {
+        if (plan_carve(c, algo, eb) != HYTG_OK) {
             why = c->err;
             continue;
         }
@@ -3109,7 +3113,7 @@ hytg_status hytg_serve_step(hytg_ctx *c, uint64_t *finished, uint64_t *busy) {
         if (c->carve.n_arrays == 0) {
             CK(cudaDeviceSynchronize());             // the last step's tasks read the old slots
             CK(ahead_drop(c));
-            s = plan_carve(c, n_arrays, c->serve_edge_budget);
+            s = plan_carve(c, algo, c->serve_edge_budget);
             if (s == HYTG_OK) s = ensure_cache(c, n_arrays);
         }
         if (s == HYTG_OK) s = ensure_second_pass(c, algo);
@@ -3272,7 +3276,7 @@ hytg_status hytg_plan(hytg_ctx *c, hytg_algo algo_in, const uint8_t *active, uin
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
     if (cap < N) return fail(c, HYTG_ERR_ARG, "output arrays too small");
     CK(cudaSetDevice(c->device));
-    hytg_status s = plan_carve(c, algo == kSSSP ? 2 : 1);
+    hytg_status s = plan_carve(c, algo);
     if (s != HYTG_OK) return s;
     std::vector<uint8_t> act_int;
     if (c->permuted) {
