@@ -1,5 +1,6 @@
 """A plan is the one of its own algorithm's run, whatever ran before, and runs
-of several algorithms in turn keep the resident partitions."""
+of several algorithms in turn keep the resident partitions: budgets that hold
+one, two and more staging slots."""
 import numpy as np
 import pytest
 
@@ -9,41 +10,43 @@ from test_gpu_parity import engine, hy  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
+BUDGETS = range(34000, 120000, 1708)
 
-def test_history(hy):
-    g = gg.rmat(13, seed=9)
-    e = engine(hy, g, g.E * 8, part_bytes=8192)
-    act = np.ones(g.V, np.uint8)
-    first = int(np.flatnonzero(np.diff(g.off.astype(np.int64)))[0])
+
+@pytest.fixture(scope="module", params=[True, False], ids=["weighted", "unweighted"])
+def eng(hy, request):
+    g = gg.random_graph(4001, 65536, seed=9, weights=request.param)
+    e = engine(hy, g, 1 << 20, part_bytes=8192)
+    e.algos = ["bfs", "pagerank"] + (["sssp"] if request.param else [])
+    yield e
+    e.close()
+
+
+def carve(e):
+    i = e.info()
+    return i["n_cached"], i["budget_used_bytes"], i["compact_edges"]
+
+
+def test_history(eng):
+    act = np.ones(eng.V, np.uint8)
 
     def plan(algo):
-        routes, counts = e.plan(algo, act)[:2]
-        i = e.info()
-        return routes.tolist(), np.asarray(counts).tolist(), i["n_cached"], i["budget_used_bytes"], i["compact_edges"]
+        routes, counts = eng.plan(algo, act)
+        return (routes.tolist(), counts.tolist(), *carve(eng))
 
-    def run(algo):
-        e.run(algo, None if algo == "pagerank" else first)
-        i = e.info()
-        return i["n_cached"], i["budget_used_bytes"], i["compact_edges"]
-
-    sizes = set()
-    for budget in range(g.E * 2, g.E * 4, g.E // 16 + 52):
-        e.set_budget(budget)
-        want = {a: plan(a) for a in ("bfs", "pagerank", "sssp")}
-        for before in ("bfs", "pagerank", "sssp"):
-            assert run(before) == want[before][2:], (budget, before)
-            for a in want:
+    for budget in BUDGETS:
+        eng.set_budget(budget)
+        want = {a: plan(a) for a in eng.algos}
+        for before in eng.algos:
+            eng.run(before, None if before == "pagerank" else 3)
+            assert carve(eng) == want[before][2:], (budget, before)
+            for a in eng.algos:
                 assert plan(a) == want[a], (budget, before, a)
-        sizes.add(want["bfs"][2])
-    assert len(sizes) > 3
 
 
-def test_cache_kept(hy):
-    g = gg.rmat(13, seed=9, weights=False)
-    e = engine(hy, g, g.E * 8, part_bytes=8192)
-    for budget in range(int(g.E * 1.5), int(g.E * 3.5), g.E // 16 + 52):
-        e.set_budget(budget)
+def test_cache_kept(eng):
+    for budget in BUDGETS:
+        eng.set_budget(budget)
         for n, algo in enumerate(["bfs", "ppr", "bfs", "ppr"]):
-            e.run(algo, 5)
-            st = e.stats()
-            assert (st["cache_fill_bytes"] > 0) == (n == 0 and e.info()["n_cached"] > 0), (budget, n)
+            eng.run(algo, 5)
+            assert (eng.stats()["cache_fill_bytes"] > 0) == (n == 0 and carve(eng)[0] > 0), (budget, n)
