@@ -33,8 +33,6 @@ __device__ __forceinline__ unsigned int sm_id() {
     return id;
 }
 
-constexpr unsigned int kInf = 0xFFFFFFFFu;
-
 // Where a task's list lies: the route's first entry and tile, its entries and
 // edges.
 struct RouteView {

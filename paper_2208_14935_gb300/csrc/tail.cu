@@ -235,11 +235,13 @@ __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThrea
         if (lane >= nl) rel = 0x7FFFFFFF;
         const long long delta = (long long)__shfl_sync(0xffffffffu, o0, from) - rel;
         const unsigned int mypay = __shfl_sync(0xffffffffu, pay, from);
-        // a resident partition's edges come from the cache unless the
-        // zero-copy route is forced
+        // a resident partition's edges come from the cache unless a forced route
+        // sends them over the link, as the body's gather and zero-copy relax read
+        // them then
         const unsigned int mypart = __shfl_sync(0xffffffffu, part, from);     // every lane, before any condition
         const unsigned int cached =
-            __ballot_sync(0xffffffffu, lane < nl && mypart < a.cp.n_cached && a.cp.force_route != kRouteZ);
+            __ballot_sync(0xffffffffu, lane < nl && mypart < a.cp.n_cached &&
+                                            (a.cp.force_route == -1 || a.cp.force_route == kRouteCache));
         // a step group's edges, targets, weights and values seen
         TailEdge ed[kTailSteps];
         int own[kTailSteps];
