@@ -184,6 +184,7 @@ struct AlgoState {
     int algo;
     unsigned int *val;       // BFS level / SSSP dist / CC label
     float *rank, *delta;     // PageRank state
+    float *rank_lo;          // what rank's roundings left out (rank_add)
     float damping, eps;
     unsigned int *bm_cur, *bm_next;
     unsigned int *overflow;  // device flag
@@ -203,6 +204,16 @@ struct AlgoState {
     unsigned long long *src_work;     // sum over entries of popcount(mask) * degree
     unsigned long long V;
 };
+// rank[v] += dl, where rank and its low part hold hi and lo.  A rank is the sum of
+// a hundred or two takes, and their roundings were the largest part of the
+// result's error (R-MAT 20, resident: 2.2e-7 in the 2-norm), more so since a
+// second pass takes hubs too; the exact error of each sum (Knuth's two-sum) is kept
+// beside it (0.5e-7; the resident run 2 % longer).
+__device__ __forceinline__ void rank_add(const AlgoState &st, unsigned long long v, float hi, float lo, float dl) {
+    const float s = hi + dl, b = s - hi;
+    st.rank[v] = s;
+    st.rank_lo[v] = lo + ((hi - (s - b)) + (dl - b));
+}
 // Edges from which a PageRank relax sums hub ids in shared memory (rank_ids).
 constexpr unsigned long long kRankNarrow = 1ull << 14, kRankWide = 1ull << 23;
 
@@ -245,6 +256,8 @@ __device__ __forceinline__ float *bmsg(const BatchState &b, unsigned long long v
     return b.msg[s >> 3] + v * kFrameSources + (s & 7);
 }
 constexpr unsigned int kHubReplicas = 256;
+// The first of them also take the block sums of k_relax_rank.
+constexpr int kRankRows = 8;
 // Batched PPR's hub copies, in the memory of the single-source replicas.
 constexpr unsigned int kBatchHubIds = 64, kBatchHubCopies = 16, kMaxPprSeeds = kMaxPprFrames * kFrameSources;
 __device__ __forceinline__ float *b_hub(const BatchState &b, unsigned int copy, unsigned int v, unsigned int s) {
@@ -408,6 +421,7 @@ cudaError_t launch_hub_reduce(const AlgoState &st, cudaStream_t s);
 cudaError_t launch_cc_jump(const AlgoState &st, unsigned long long n_words_alloc, cudaStream_t s);
 cudaError_t launch_cc_final(const AlgoState &st, unsigned long long V, unsigned int *tmp,
                             unsigned int *out, cudaStream_t s);
+cudaError_t launch_pr_rank(const AlgoState &st, unsigned long long V, float *out, cudaStream_t s);
 cudaError_t launch_to_original(const unsigned int *perm, const unsigned int *in, float *out,
                                unsigned long long V, cudaStream_t s);
 cudaError_t launch_upload_bitmap(const unsigned char *active_dev, unsigned int *bm,

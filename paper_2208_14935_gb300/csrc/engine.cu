@@ -260,6 +260,7 @@ struct hytg_ctx {
     unsigned int *d_perm = nullptr;
     float *d_hub_rep = nullptr;                          // kHubReplicas x n_hub_rep floats
     unsigned int n_hub_rep = 0;
+    float *d_rank_lo = nullptr;                          // low parts of the ranks, made by the first PageRank or PPR run
 
     // batched runs (several sources in one run, sharing every transfer)
     BatchState bs{};
@@ -591,7 +592,7 @@ void free_graph(hytg_ctx *c) {
     dfree(c->d_off); dfree(c->d_val); dfree(c->d_delta); dfree(c->d_bm[0]); dfree(c->d_bm[1]);
     dfree(c->d_out); dfree(c->d_ebase); dfree(c->d_soff); dfree(c->d_pay); dfree(c->d_tiles);
     dfree(c->d_part_wb); dfree(c->d_part_eb); dfree(c->d_sumbuf); dfree(c->d_perm); dfree(c->d_round_part);
-    dfree(c->d_hub_rep);
+    dfree(c->d_hub_rep); dfree(c->d_rank_lo);
     dfree(c->d_sp_ebase); dfree(c->d_sp_soff); dfree(c->d_sp_pay64); dfree(c->d_sp_vid);
     dfree(c->d_sp_cursor); dfree(c->d_sp_tiles);
     c->n_hub_rep = 0;
@@ -1099,6 +1100,7 @@ AlgoState algo_state(hytg_ctx *c, int algo, unsigned int bucket_limit = 0xFFFFFF
     st.algo = algo;
     st.val = c->d_val;
     st.rank = (float *)c->d_val;
+    st.rank_lo = c->d_rank_lo;
     st.delta = c->d_delta;
     st.damping = (float)c->pr_damping;
     st.eps = (float)c->pr_eps;
@@ -2551,6 +2553,8 @@ hytg_status hytg_load_csr(hytg_ctx *c, uint64_t V, uint64_t E, const uint64_t *o
             CK(cudaMalloc(&c->d_perm, V * 4));
             CK(cudaMemcpy(c->d_perm, c->h_perm.data(), V * 4, cudaMemcpyHostToDevice));
             c->n_hub_rep = (unsigned int)std::min<uint64_t>(c->n_hubs, (uint64_t)c->hub_replicas);
+            // replica rows start on 16 bytes: k_relax_rank adds four ids at once
+            if (c->n_hub_rep > 4) c->n_hub_rep &= ~3u;
             if (c->n_hub_rep) {
                 CK(cudaMalloc(&c->d_hub_rep, (size_t)kHubReplicas * c->n_hub_rep * 4));
                 CK(cudaMemset(c->d_hub_rep, 0, (size_t)kHubReplicas * c->n_hub_rep * 4));
@@ -2767,6 +2771,7 @@ hytg_status hytg_run(hytg_ctx *c, hytg_algo algo_in, const uint32_t *sources, ui
         s = ensure_cache(c, n_arrays);
         if (s == HYTG_OK) s = ensure_second_pass(c, algo);
         if (s != HYTG_OK) return s;
+        if ((algo == kPR || algo == kPPR) && c->batch_mode == kBatchNone) ENSURE(c->d_rank_lo, c->V * 4);
         // delta-stepping bucket (SSSP only): eligible vertices have dist < bucket
         uint64_t delta = 0;
         if (algo == kSSSP && c->batch_mode == kBatchNone)
@@ -3212,7 +3217,7 @@ hytg_status hytg_fetch_pagerank_state(hytg_ctx *c, float *rank, float *delta, ui
     CK(cudaSetDevice(c->device));
     // original vertex order; d_out (the normalised result) is rebuilt afterwards
     if (rank) {
-        CK(launch_to_original(c->d_perm, c->d_val, c->d_out, c->V, c->s_main));
+        CK(launch_pr_rank(algo_state(c, c->last_algo), c->V, c->d_out, c->s_main));
         CK(cudaMemcpyAsync(rank, c->d_out, c->V * 4, cudaMemcpyDeviceToHost, c->s_main));
     }
     if (delta) {
@@ -3247,7 +3252,7 @@ hytg_status hytg_get_info(hytg_ctx *c, hytg_info *out) {
     i.budget_bytes = c->budget;
     i.budget_used_bytes = c->carve.used;
     i.compact_edges = c->carve.compact_edges;
-    i.vertex_state_bytes = c->loaded ? c->vertex_bytes + second_pass_bytes(c) : 0;
+    i.vertex_state_bytes = c->loaded ? c->vertex_bytes + second_pass_bytes(c) + (c->d_rank_lo ? c->V * 4 : 0) : 0;
     i.pinned_host_bytes = c->loaded ? 4 * (packed_words(c->E, c->dst_bits) +
                                            (c->weighted ? packed_words(c->E, c->w_bits) : 0)) : 0;
     *out = i;

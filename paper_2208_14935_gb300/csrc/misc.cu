@@ -20,10 +20,10 @@ __global__ void k_init(AlgoState st, unsigned long long V, unsigned long long n_
             case kBFS:
             case kSSSP: st.val[v] = (v == source) ? 0u : 0xFFFFFFFFu; break;
             case kCC: st.val[v] = (unsigned int)v; break;   // internal id, mapped at the end
-            case kPR: st.rank[v] = 0.0f; st.delta[v] = base; break;
+            case kPR: st.rank[v] = st.rank_lo[v] = 0.0f; st.delta[v] = base; break;
             // PPR: the seed holds the whole initial residual of PageRank,
             // (1 - d) V, so that eps bounds the same relative error
-            default: st.rank[v] = 0.0f; st.delta[v] = (v == source) ? base * (float)V : 0.0f; break;
+            default: st.rank[v] = st.rank_lo[v] = 0.0f; st.delta[v] = (v == source) ? base * (float)V : 0.0f; break;
         }
     }
     const bool all = (st.algo == kCC || st.algo == kPR);
@@ -158,7 +158,7 @@ __global__ void k_pr_sums(AlgoState st, unsigned long long V, double *sums) {
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long v = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; v < V;
          v += stride) {
-        r += st.rank[v];
+        r += (double)st.rank[v] + st.rank_lo[v];
         d += fabs((double)st.delta[v]);
     }
 #pragma unroll
@@ -188,7 +188,14 @@ __global__ void k_pr_normalise(AlgoState st, unsigned long long V, const double 
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long v = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; v < V;
          v += stride)
-        out[st.perm ? st.perm[v] : v] = (float)((double)st.rank[v] * inv);
+        out[st.perm ? st.perm[v] : v] = (float)(((double)st.rank[v] + st.rank_lo[v]) * inv);
+}
+
+// The ranks before they are normalised, in original vertex order.
+__global__ void k_pr_rank(AlgoState st, unsigned long long V, float *out) {
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long v = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; v < V; v += stride)
+        out[st.perm ? st.perm[v] : v] = st.rank[v] + st.rank_lo[v];
 }
 
 // Copy a per-vertex array from internal to original vertex order.
@@ -400,6 +407,11 @@ cudaError_t launch_pr_frontier(const AlgoState &st, unsigned long long V,
     unsigned long long g = (n + 255) / 256;
     if (g > 16ull * device_sms()) g = 16ull * device_sms();
     k_pr_frontier<<<(unsigned int)g, 256, 0, s>>>(st, V, n_words_alloc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pr_rank(const AlgoState &st, unsigned long long V, float *out, cudaStream_t s) {
+    k_pr_rank<<<grid_for(V, 256), 256, 0, s>>>(st, V, out);
     return cudaGetLastError();
 }
 

@@ -451,20 +451,24 @@ __global__ void __launch_bounds__(256) k_bin(GraphDev g, AlgoState st, PartArray
         unsigned int elig[4];
         unsigned long long o0[4], deg[4];
         unsigned int vv[4];
-        float rk[4];
+        float rk[4], rl[4];
         unsigned long long bf[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             o0[q] = deg[q] = 0;
             vv[q] = 0;
-            rk[q] = 0.0f;
+            rk[q] = rl[q] = 0.0f;
             bf[q] = 0;
             if ((wq[q] >> lane) & 1u) {
                 const unsigned long long v = (unsigned long long)(w0 + q) * 32 + lane;
                 o0[q] = g.off[v];
                 deg[q] = g.off[v + 1];
                 if (MODE == kBinBatch) bf[q] = st.batch_mode == kBatchPPR ? st.b_fr32[v] : st.b_fr[v];
-                else if (MODE == kBinPR) { vv[q] = __float_as_uint(st.delta[v]); rk[q] = st.rank[v]; }
+                else if (MODE == kBinPR) {
+                    vv[q] = __float_as_uint(st.delta[v]);
+                    rk[q] = st.rank[v];
+                    rl[q] = st.rank_lo[v];
+                }
                 else vv[q] = st.val[v];
             }
         }
@@ -540,7 +544,7 @@ __global__ void __launch_bounds__(256) k_bin(GraphDev g, AlgoState st, PartArray
                         const unsigned long long v = (unsigned long long)(w0 + q) * 32 + lane;
                         const float dl = __uint_as_float(vv[q]);
                         st.delta[v] = 0.0f;
-                        st.rank[v] = rk[q] + dl;
+                        rank_add(st, v, rk[q], rl[q], dl);
                         vv[q] = __float_as_uint(deg[q] ? st.damping * dl / (float)deg[q] : 0.0f);
                     }
                 }

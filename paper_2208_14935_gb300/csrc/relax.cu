@@ -96,13 +96,19 @@ __global__ void __launch_bounds__(kRelaxBlock, 3) k_relax(AlgoState st, ListArra
 // 140 to 165 with R-MAT's in-degree skew and per-SM replicas of 4,096 hub ids.
 // Hub sorting puts the hottest targets at the lowest ids, so a block of 1,024
 // threads (one per SM) sums the pushes to ids below ns in shared memory and adds
-// the sums to delta at its end, four ids per vector reduction; a probe with the
+// the sums to memory at its end, four ids per vector reduction; a probe with the
 // skew of 2^20 / 2^24 vertices then runs at 261 / 221 G pushes/s (ns = 16,384)
 // against 137 / 166 with the replicas, and the relax of R-MAT 24's cache, 157 M
-// edges, at 240 G pushes/s against 94.  delta also holds the hubs' residuals
-// once the launch ends, where a second pass finds them (replicas are folded
-// once per iteration): R-MAT 20, resident, 71 iterations instead of 97.  Whole
-// runs: 22.5 -> 15 ms there, PPR on R-MAT 24 238 -> 210 ms.  TB: a second,
+// edges, at 240 G pushes/s against 94.  The sums go to kRankRows rows of the hub
+// replicas in turn (ids beyond the replicas: to delta), which a second pass adds
+// to the residuals that it looks at (k_sp_take), as the end of the iteration adds
+// all replicas: R-MAT 20, resident, 71 iterations instead of 97.  Whole runs:
+// 22.5 -> 16 ms there, PPR on R-MAT 24 238 -> 210 ms.  The rows are for the
+// rounding: with F tasks and their second passes an iteration has tens of
+// launches, each of 152 or 304 blocks, and thousands of additions to one running
+// 32-bit sum per hub doubled the result's error (PageRank, R-MAT 19 in 32
+// partitions at a budget of 30 %: 1.9e-7 with the replicas, 4.6e-7 with sums into
+// delta, 2.7e-7 with eight rows; with rank_add's low parts 0.8e-7).  TB: a second,
 // device-sized task in the same launch.
 //
 // The kRankHot hottest ids have a sum per lane: an addition to shared memory is
@@ -157,10 +163,11 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_relax_rank(AlgoState st
         if ((threadIdx.x & 31) == 0) acc[v] = x;    // ids below kRankHot have no other sum
     }
     __syncthreads();
+    float4 *row = reinterpret_cast<float4 *>(st.hub_rep + (size_t)(blockIdx.x % kRankRows) * st.n_hub_rep);
     for (unsigned int i = threadIdx.x; i < ns / 4; i += BLOCK) {
         const float4 x = acc4[i];
         if (x.x != 0.f || x.y != 0.f || x.z != 0.f || x.w != 0.f)
-            atomicAdd(reinterpret_cast<float4 *>(st.delta) + i, x);
+            atomicAdd(i < st.n_hub_rep / 4 ? row + i : reinterpret_cast<float4 *>(st.delta) + i, x);
     }
 }
 
@@ -248,6 +255,37 @@ __global__ void __launch_bounds__(kRelaxBlock) k_sp_take(AlgoState st, const uns
         float dl[4];
         unsigned int pay[4];
         unsigned long long o0[4], deg[4];
+        float hub[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (ALGO == kPR && b0 < st.n_hub_rep) {     // block-uniform
+            // the hubs' block sums (k_relax_rank) join their residuals.  What a row
+            // gave is taken off it by a reduction, as from delta below, so that
+            // other streams' sums stay; all of a lane's loads are in flight
+            // together (swapping the rows out waits for each: +7 % of a resident
+            // R-MAT 20 PageRank, this +0.3 %).
+            float x[4][kRankRows];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned long long v = v0 + 32 * q + lane;
+                const bool in = v < r.vhi && v < st.n_hub_rep;
+#pragma unroll
+                for (int k = 0; k < kRankRows; ++k)
+                    x[q][k] = in ? __ldcg(&st.hub_rep[(size_t)k * st.n_hub_rep + v]) : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int k = 0; k < kRankRows; ++k)
+                    if (x[q][k] != 0.0f)
+                        atomicAdd(&st.hub_rep[(size_t)k * st.n_hub_rep + (v0 + 32 * q + lane)], -x[q][k]);
+#pragma unroll
+            for (int w = kRankRows / 2; w > 0; w >>= 1)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int k = 0; k < w; ++k) x[q][k] += x[q][k + w];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) hub[q] = x[q][0];
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const unsigned long long v = v0 + 32 * q + lane;
@@ -256,7 +294,8 @@ __global__ void __launch_bounds__(kRelaxBlock) k_sp_take(AlgoState st, const uns
             pay[q] = 0;
             if (v < r.vhi) {
                 if (ALGO == kPR) {
-                    dl[q] = __ldcg(&st.delta[v]);
+                    if (v < st.n_hub_rep && hub[q] != 0.0f) dl[q] = atomicAdd(&st.delta[v], hub[q]) + hub[q];
+                    else dl[q] = __ldcg(&st.delta[v]);
                     take[q] = dl[q] > st.eps;
                 } else {
                     take[q] = (__ldcg(&st.bm_cur[v >> 5]) >> (v & 31)) & 1u;
@@ -288,7 +327,7 @@ __global__ void __launch_bounds__(kRelaxBlock) k_sp_take(AlgoState st, const uns
                     // one, so this thread is the only writer of rank[v] now: a
                     // plain update suffices.
                     atomicAdd(&st.delta[v], -dl[q]);
-                    st.rank[v] += dl[q];
+                    rank_add(st, v, st.rank[v], st.rank_lo[v], dl[q]);
                     if (deg[q]) pay[q] = __float_as_uint(st.damping * dl[q] / (float)deg[q]);
                 } else if (st.bucket_limit != 0xFFFFFFFFu && pay[q] >= st.bucket_limit) {
                     deg[q] = 0;

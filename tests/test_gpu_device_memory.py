@@ -28,7 +28,7 @@ def refused(hy, call):
     assert ex.value.status == hy.HYTG_ERR_CUDA and "device allocation" in str(ex.value)
 
 
-@pytest.mark.parametrize("name", SECOND_PASS)
+@pytest.mark.parametrize("name", SECOND_PASS + ["d_rank_lo"])
 @pytest.mark.parametrize("algo", ["pagerank", "ppr"])
 def test_second_pass(hy, e, monkeypatch, name, algo):
     before = e.info()["vertex_state_bytes"]
@@ -40,7 +40,7 @@ def test_second_pass(hy, e, monkeypatch, name, algo):
     check(e.graph, algo, e.run(algo, src), src)
     info = e.info()
     n = info["n_parts"]
-    assert info["vertex_state_bytes"] - before == e.V * 16 + (e.graph.E // 2048 + n + 2) * 4 + n * 8
+    assert info["vertex_state_bytes"] - before == e.V * 20 + (e.graph.E // 2048 + n + 2) * 4 + n * 8
 
 
 @pytest.mark.parametrize("name", SECOND_PASS + ["d_sp_pay64", "d_sp_vid", "d_pay64", "d_vid", "d_bout", "bs.fr32", "frame"])
