@@ -384,13 +384,17 @@ cudaError_t launch_second_pass(const AlgoState &st, const unsigned long long *of
 }
 
 // Hub ids that a PageRank relax of at most `edges` edges sums in shared memory,
-// a multiple of 4; 0: the plain relax with replicas.  A block's sums cost its
-// share of the flush (a vector reduction per 4 ids), so the number follows the
-// edges an SM gets.  PageRank, every partition resident, plain / 4,096 / 16,384:
-// R-MAT 18 (4.2 M edges) 8.0 / 6.4 / 6.9 ms, R-MAT 19 13.1 / 11.0 / 9.3, R-MAT 21
-// 37.0 / - / 27.4; R-MAT 12 (65 K edges) 5.4 / 3.2.
+// a multiple of 4; 0: the plain relax.  Of hub-sorted graphs, with or without
+// replicas ("hub_replicas" 0: every sum goes to delta; one addition per edge there
+// gave R-MAT 19, resident, an error of 3.8e-6, 152 sums a launch 0.7e-7).  A
+// block's sums cost its share of the flush (a vector reduction per 4 ids), so the
+// number follows the edges an SM gets.  PageRank, every partition resident, plain
+// / 4,096 / 16,384: R-MAT 18 (4.2 M edges) 8.0 / 6.4 / 6.9 ms, R-MAT 19 13.1 / 11.0
+// / 9.3, R-MAT 21 37.0 / - / 27.4; R-MAT 12 (65 K edges) 5.4 / 3.2.  The edges of a
+// device-sized launch are those of its source, since the host does not know the
+// route's: a late iteration with few edges clears and scans the sums all the same.
 static unsigned int rank_ids(const AlgoState &st, unsigned long long edges) {
-    if ((st.algo != kPR && st.algo != kPPR) || !st.hub_rep || st.V < 4 * kRankHot || edges < kRankNarrow) return 0;
+    if ((st.algo != kPR && st.algo != kPPR) || !st.perm || st.V < 4 * kRankHot || edges < kRankNarrow) return 0;
     if (edges >= kRankWide && st.V >= 16384) return 16384;
     return st.V >= 4096 ? 4096u : (unsigned int)st.V & ~3u;
 }
