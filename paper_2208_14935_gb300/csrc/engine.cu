@@ -299,6 +299,7 @@ struct hytg_ctx {
     uint32_t serve_frames_used = 0;                      // bit f: frame f attached to a group
     int serve_group_frame[kMaxFrames] = {};              // frame of each group of 8 slots, or -1
     uint64_t serve_edge_budget = 0;
+    bool serve_lost = false;                             // the open session's graph, pool or frontier is gone
 
     // partitions
     uint64_t part_edges = 0, max_part_edges = 0;
@@ -434,6 +435,8 @@ namespace {
 const char *kStatusStr[] = {"ok", "invalid argument", "CUDA error", "device budget too small",
                             "pinned host allocation failed", "SSSP distance overflow",
                             "device wait timed out", "call out of order"};
+
+const char *kServeLost = "hytg_load_csr, hytg_set_device_budget or hytg_plan took the session's state (hytg_serve_end first)";
 
 hytg_status fail(hytg_ctx *c, hytg_status s, const std::string &msg) {
     if (c) c->err = msg;
@@ -603,6 +606,7 @@ void free_graph(hytg_ctx *c) {
     for (auto &f : c->own_ppr) dfree(f);
     c->bs = BatchState{};
     c->batch_mode = kBatchNone;
+    c->serve_lost = c->serving;
     c->permuted = false;
     c->n_hubs = 0;
     c->h_perm.clear();
@@ -2593,6 +2597,7 @@ hytg_status hytg_set_device_budget(hytg_ctx *c, uint64_t bytes) {
     if (!c) return HYTG_ERR_ARG;
     CK(cudaSetDevice(c->device));
     CK(cudaDeviceSynchronize());
+    c->serve_lost = c->serving;
     dfree(c->d_pool);
     c->budget = 0;
     c->carve = Carve();
@@ -3069,6 +3074,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
     CK(cudaMemsetAsync(c->d_report, 0, offsetof(RunReport, sp), c->s_main));
     CK(launch_b_init(c->bs, c->V, c->n_words_alloc, c->d_src, 0, 0.0f, c->d_bm[0], c->s_main));
     c->serving = true;
+    c->serve_lost = false;
     c->serve_algo = algo;
     c->serve_it = 0;
     c->serve_busy = 0;
@@ -3079,6 +3085,7 @@ hytg_status hytg_serve_begin(hytg_ctx *c, hytg_algo algo_in, uint32_t n_slots) {
 hytg_status hytg_serve_admit(hytg_ctx *c, uint32_t slot, uint32_t source) {
     if (!c) return HYTG_ERR_ARG;
     if (!c->serving) return fail(c, HYTG_ERR_STATE, "not serving");
+    if (c->serve_lost) return fail(c, HYTG_ERR_STATE, kServeLost);
     if (slot >= c->batch_K) return fail(c, HYTG_ERR_ARG, "slot out of range");
     if (c->serve_busy & (1ull << slot)) return fail(c, HYTG_ERR_STATE, "slot is busy");
     if (source >= c->V) return fail(c, HYTG_ERR_ARG, "source out of range");
@@ -3107,6 +3114,7 @@ hytg_status hytg_serve_admit(hytg_ctx *c, uint32_t slot, uint32_t source) {
 hytg_status hytg_serve_step(hytg_ctx *c, uint64_t *finished, uint64_t *busy) {
     if (!c) return HYTG_ERR_ARG;
     if (!c->serving) return fail(c, HYTG_ERR_STATE, "not serving");
+    if (c->serve_lost) return fail(c, HYTG_ERR_STATE, kServeLost);
     CK(cudaSetDevice(c->device));
     try {
         const int algo = c->serve_algo;
@@ -3146,6 +3154,7 @@ hytg_status hytg_serve_step(hytg_ctx *c, uint64_t *finished, uint64_t *busy) {
 hytg_status hytg_serve_fetch(hytg_ctx *c, uint32_t slot, void *out, uint64_t out_bytes) {
     if (!c || !out) return HYTG_ERR_ARG;
     if (!c->serving) return fail(c, HYTG_ERR_STATE, "not serving");
+    if (c->serve_lost) return fail(c, HYTG_ERR_STATE, kServeLost);
     if (slot >= c->batch_K) return fail(c, HYTG_ERR_ARG, "slot out of range");
     const uint64_t bit = 1ull << slot;
     if (!(c->serve_busy & bit) || (c->serve_alive & bit))
@@ -3281,6 +3290,7 @@ hytg_status hytg_plan(hytg_ctx *c, hytg_algo algo_in, const uint8_t *active, uin
     const uint32_t N = (uint32_t)(c->part_vb.size() - 1);
     if (cap < N) return fail(c, HYTG_ERR_ARG, "output arrays too small");
     CK(cudaSetDevice(c->device));
+    c->serve_lost = c->serve_lost || c->serving;     // its carve and frontier are used here
     hytg_status s = plan_carve(c, algo);
     if (s != HYTG_OK) return s;
     std::vector<uint8_t> act_int;

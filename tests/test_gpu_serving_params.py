@@ -52,3 +52,37 @@ def test_set_between_steps(hy, g, algo, changes):
             x, _, _ = orc.pagerank(g, tol=1e-13, seed=src[k])
             assert float(np.abs(got.astype(np.float64) - x).sum()) <= PR_TOL
     e.close()
+
+
+@pytest.mark.parametrize("replace", ["graph", "budget", "frontier"])
+@pytest.mark.parametrize("algo", ["ppr", "bfs"])
+def test_replaced_under_a_session(hy, g, algo, replace):
+    """A session whose graph, device budget or frontier is replaced can only be
+    closed."""
+    budget = g.E * 8 + g.V * 96 * 2 + (1 << 17)
+    e = hy.Engine(g, budget=budget, params={"part_bytes": 16384})
+    a = hy.ALGOS[algo]
+    hy.hytg_serve_begin(e.ctx, a, 2)
+    hy.hytg_serve_admit(e.ctx, 0, 3)
+    hy.hytg_serve_step(e.ctx)
+    if replace == "frontier":
+        e.plan(algo, np.ones(g.V, np.uint8))
+    else:
+        e.load(g) if replace == "graph" else e.set_budget(budget)
+    for call in (lambda: hy.hytg_serve_step(e.ctx), lambda: hy.hytg_serve_admit(e.ctx, 1, 4),
+                 lambda: hy.hytg_serve_fetch(e.ctx, 0, g.V, a)):
+        with pytest.raises(hy.HytgError) as ex:
+            call()
+        assert ex.value.status == hy.HYTG_ERR_STATE
+    hy.hytg_serve_end(e.ctx)
+    hy.hytg_serve_begin(e.ctx, a, 2)
+    hy.hytg_serve_admit(e.ctx, 0, 3)
+    while not hy.hytg_serve_step(e.ctx)[0] & 1:
+        pass
+    got = hy.hytg_serve_fetch(e.ctx, 0, g.V, a)
+    hy.hytg_serve_end(e.ctx)
+    if algo == "bfs":
+        assert np.array_equal(got, orc.bfs(g, 3)[0])
+    else:
+        assert float(np.abs(got.astype(np.float64) - orc.pagerank(g, tol=1e-13, seed=3)[0]).sum()) <= PR_TOL
+    e.close()
