@@ -584,9 +584,10 @@ def main():
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     roofline, roofline_l2 = None, None
     if not args.no_timing and "pagerank" in algos:
-        # PageRank is most of the step; its two heaviest kernels are the second
-        # pass over resident partitions and the F-route relax.  Per launch from
-        # the timeline (CUDA events on the launching stream, timed region only).
+        # PageRank is most of the step; its two heaviest parts are the second
+        # pass over resident partitions (k_sp_take, then k_relax_rank on its list)
+        # and the F-route relax (k_relax_rank).  Per launch from the timeline (CUDA
+        # events on the launching stream, timed region only).
         tls = [p["pagerank"]["tl"] for p in steps]
         prs = [p["pagerank"]["stats"] for p in steps]
         sp_n, sp_ms = sum(t["sp_n"] for t in tls), sum(t["sp_ms"] for t in tls)
@@ -598,25 +599,28 @@ def main():
         kern = {}
         if sp_n:
             # per relaxed edge its packed target + 8 B value read-modify-write; per
-            # scanned vertex 16 B offsets, 4 B delta read, 8 B delta and rank updates
-            kern["k_second_pass<PageRank>"] = (sp_n, sp_ms, sp_e, sp_e * (eb + 8) + sp_v * 28,
-                                               f"per edge {eb} + 8 (value RMW), per scanned vertex 28",
-                                               sp_v)
+            # scanned vertex 16 B offsets, 4 B delta read, 12 B delta and rank updates
+            kern["second pass: k_sp_take + k_relax_rank"] = (
+                sp_n, sp_ms, sp_e, sp_e * (eb + 8) + sp_v * 32,
+                f"per edge {eb} + 8 (value RMW), per scanned vertex 32", sp_v)
         if rf_n:
             # per edge its packed target + 8 B RMW, per list entry 20 B
-            kern["k_relax<PageRank> F route"] = (rf_n, rf_ms, rf_e, rf_e * (eb + 8) + rf_v * 20,
-                                                 f"per edge {eb} + 8 (value RMW), per active vertex 20",
-                                                 rf_v)
+            kern["F route: k_relax_rank"] = (rf_n, rf_ms, rf_e, rf_e * (eb + 8) + rf_v * 20,
+                                             f"per edge {eb} + 8 (value RMW), per active vertex 20", rf_v)
         if kern:
             dom = max(kern, key=lambda k: kern[k][1])
             n, ms, e_, alg, model, vv = kern[dom]
             achieved = alg / (ms * 1e-3) / 1e9
-            # DRAM bytes of both kernels' relax from one ncu capture of its dense
-            # launch on R-MAT 22: 245.7 MB for 67,108,864 edges; scaled to this
-            # run's mean launch by its edges
-            traffic = 245730048 / 67108864 * (e_ / n)
-            note = ("scaled from an ncu capture of k_relax_rank on R-MAT 22 (3.66 B/edge) by this run's "
-                    "edges per launch" + (", without the take" if dom.startswith("k_second_pass") else ""))
+            # DRAM bytes from an ncu capture of dense launches on R-MAT 22: the
+            # relax moves 1.10 of its edges' packed bits and 20 B per list entry
+            # (245.9 MB for 67,108,864 edges of 22 bits in 2,009,398 lists), the take
+            # 23.9 B per scanned vertex (100.3 MB for 4,194,304)
+            traffic = 1.10 * (eb * e_ + 20 * vv) / n
+            note = ("modelled from an ncu capture on R-MAT 22: 1.10 x (packed edge + 20 B per list entry) of the "
+                    "relax")
+            if dom.startswith("second pass"):
+                traffic += 23.9 * vv / n
+                note += " + 23.9 B per scanned vertex of the take; at most, since not every scanned vertex is listed"
             roofline = {"kernel": dom, "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                         "frac": achieved / hbm, "traffic": traffic, "traffic_note": note,
                         "bytes_model": model, "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_src})",
@@ -631,8 +635,9 @@ def main():
                     roofline_l2[k] = {"bound": "l2_reductions", "achieved": rate, "peak": peak,
                                       "unit": "G updates/s", "frac": rate / peak,
                                       "frac_of_uniform_probe": rate / red_probe[0]}
-                roofline_l2["peak_source"] = ("hytg_probe_atomics_hub in this run: the R-MAT in-degree "
-                                              "skew after hub sorting, with the kernels' per-SM replicas")
+                roofline_l2["peak_source"] = ("hytg_probe_atomics_hub in this run: the R-MAT in-degree skew after "
+                                              "hub sorting, every push reduced in L2, hub ids in per-SM replicas; "
+                                              "k_relax_rank sums hub ids on chip, so this is no bound for it")
                 roofline_l2["uniform_gops"] = red_probe[0]
                 roofline_l2["skewed_gops"] = red_probe[1]
                 roofline_l2["hub_skew_without_replicas_gops"] = hub_probe[0]

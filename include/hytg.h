@@ -309,8 +309,8 @@ hytg_status hytg_fetch_result(hytg_ctx *ctx, void *out, uint64_t out_bytes);
  * host threads of the context fault in the pages of `out`, with a store to
  * each, while the run is on the device, so that the copy does not take the
  * page faults of a fresh allocation one at a time.  `out` must stay valid
- * until the call returns; after an error its first 4*V*n_sources bytes are
- * undefined.  Arguments and errors are those of the two calls. */
+ * until the call returns and must not overlap `sources`; after an error its
+ * first 4*V*n_sources bytes are undefined.  Arguments and errors are those of the two calls. */
 hytg_status hytg_run_fetch(hytg_ctx *ctx, hytg_algo algo, const uint32_t *sources, uint32_t n_sources,
                            void *out, uint64_t out_bytes);
 
@@ -436,7 +436,10 @@ hytg_status hytg_get_timeline(hytg_ctx *ctx, hytg_timed_launch *out, uint32_t ca
  * normalised to sum 1) and frees the slot; hytg_serve_end closes the run.
  * Queries admitted while others are running join them at the next
  * iteration, so their work overlaps on the device; a query's result does not
- * depend on the others.  hytg_run is refused while serving. */
+ * depend on the others.  hytg_run is refused while serving.  Parameters may be
+ * set between steps; hytg_load_csr, hytg_set_device_budget and hytg_plan take
+ * the session's state, after which its calls return HYTG_ERR_STATE until
+ * hytg_serve_end. */
 hytg_status hytg_serve_begin(hytg_ctx *ctx, hytg_algo algo, uint32_t n_slots);
 /* hytg_serve_admit: HYTG_ERR_BUDGET when the slot's group of 8 has no frame
  * of device memory and none is free (see hytg_serve_get_info). */

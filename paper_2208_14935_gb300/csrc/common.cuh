@@ -11,7 +11,7 @@ constexpr int kRoutes = 5;            // NONE, CACHE, F, C, Z (hytg_route)
 constexpr int kRouteNone = 0, kRouteCache = 1, kRouteF = 2, kRouteC = 3, kRouteZ = 4;
 
 // Frontier bitmap: one bit per vertex, 32-bit words, padded to a multiple of
-// 32 words; the planning kernels walk it one 32-word round per warp.  One
+// 32 words; the planning kernels walk it in units of four words (plan.cu).  One
 // bitmap serves a whole run: k_bin clears the bits it takes, the relax
 // kernels set the bits of changed vertices for the next iteration.
 constexpr int kBitmapPadWords = 32;
@@ -190,8 +190,10 @@ struct AlgoState {
     unsigned int *overflow;  // device flag
     unsigned int n_arrays;   // edge arrays read per edge (1 or 2)
     const unsigned int *perm;// internal id -> original id (hub sorting), or nullptr
-    // PageRank pushes to hub ids [0, n_hub_rep) go to per-SM replicas
-    // hub_rep[(smid % kHubReplicas) * n_hub_rep + v], summed into delta once per iteration
+    // PageRank pushes to hub ids [0, n_hub_rep) go to replica rows of n_hub_rep sums:
+    // a plain relax adds each to its SM's row (smid % kHubReplicas), k_relax_rank
+    // its blocks' sums to the first kRankRows; all rows join delta once per
+    // iteration, those first ones also when a second pass looks at their ids
     float *hub_rep;
     unsigned int n_hub_rep;
     unsigned int bucket_limit;  // SSSP delta-stepping: only dist < limit is eligible (~0u: off)
@@ -256,7 +258,7 @@ __device__ __forceinline__ float *bmsg(const BatchState &b, unsigned long long v
     return b.msg[s >> 3] + v * kFrameSources + (s & 7);
 }
 constexpr unsigned int kHubReplicas = 256;
-// The first of them also take the block sums of k_relax_rank.
+// The first of them also take the block sums of k_relax_rank, in turn.
 constexpr int kRankRows = 8;
 // Batched PPR's hub copies, in the memory of the single-source replicas.
 constexpr unsigned int kBatchHubIds = 64, kBatchHubCopies = 16, kMaxPprSeeds = kMaxPprFrames * kFrameSources;

@@ -865,7 +865,9 @@ hytg_status plan_carve(hytg_ctx *c, int algo, uint64_t edge_budget = 0) {
     // 1.91 / 1.43 ms; 64-source BFS 3.03 / 2.75; PageRank 40 / 29 ms.  PageRank
     // and PPR keep larger tasks when the slots are small: a copy of a few MB is
     // short beside the relax and second pass, which then only become more and
-    // smaller launches (32-seed PPR on R-MAT 18, 2.4 MB: 48 / 53 ms).
+    // smaller launches (32-seed PPR on R-MAT 18, 2.4 MB: 48 / 53 ms).  The line of
+    // 8 MB lies between that and the PageRank above (9.4 MB); nothing between
+    // them was measured.
     const bool rank = algo == kPR || algo == kPPR;
     const uint64_t region = n_slots * bytes(slot_edges);
     if (n_slots < 3 && (!rank || region >= (8u << 20))) {
@@ -1486,8 +1488,10 @@ bool loop_applies(const hytg_ctx *c) {
 // slot; the host combines partitions into tasks and overlaps them on several
 // streams.  A 32-seed PPR has about a hundred F iterations: in the loop against
 // from the host, R-MAT 16 44 / 30 ms, R-MAT 18 78 / 47 ms, R-MAT 20 194 / 156 ms.
-// Batched BFS and SSSP have two or three, and their option promises the loop
-// (R-MAT 20 3.0 against 2.4 ms), as it does for small PPR.
+// Batched BFS and SSSP have two or three (R-MAT 20 3.0 against 2.4 ms).  So the
+// host is the faster path at every size measured, R-MAT 16 at the line itself
+// included; below it, and for BFS and SSSP, the loop is kept for what
+// "device_loop" 1 promises a caller (no host work per iteration), not for speed.
 constexpr uint64_t kLoopFcEdges = 1u << 20;
 bool loop_fc_wanted(const hytg_ctx *c) {
     if (c->device_loop < 2 &&

@@ -19,7 +19,8 @@ namespace hytg {
 namespace {
 
 // cur: v's value, read shortly before (BFS, SSSP, CC); hub_rep: this SM's
-// replica row of the hub accumulators (PageRank only).
+// replica row of the hub accumulators (PageRank only: launches with too few edges
+// for k_relax_rank, and the zero-copy route's).
 template <int ALGO>
 __device__ __forceinline__ void relax_edge(const AlgoState &st, unsigned int v, unsigned int pay,
                                            unsigned int w, unsigned int cur, float *hub_rep) {
@@ -27,8 +28,8 @@ __device__ __forceinline__ void relax_edge(const AlgoState &st, unsigned int v, 
         // fire-and-forget reduction; the next frontier is rebuilt from delta
         // (delta > eps) by k_pr_frontier once every relax of the iteration is
         // done.  Pushes to the hottest vertices (hub-sorted ids below
-        // n_hub_rep) go to this SM's replica, so thousands of SMs' updates do
-        // not serialise on one L2 address.
+        // n_hub_rep) go to this SM's replica, so that the SMs' updates do not
+        // serialise on one L2 address.
         if (v < st.n_hub_rep) atomicAdd(&hub_rep[v], __uint_as_float(pay));
         else atomicAdd(&st.delta[v], __uint_as_float(pay));
     } else {
